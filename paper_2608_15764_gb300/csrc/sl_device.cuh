@@ -100,11 +100,15 @@ __device__ __forceinline__ float fp8_word_sum(uint32_t w, float acc) {
 // 256-thread (two 512-thread) CTAs stay resident: with fewer warps its
 // dependent TwoSum chains cannot hide the load latency (at K = 8 the
 // unconstrained allocation of 78 registers leaves three CTAs and ~7% less
-// bandwidth).  Every other kernel takes the registers it wants (K loaded
-// vectors must stay in registers).
+// bandwidth).  A K = 1 kernel of another type is held to the 32 registers that
+// let an SM's 2,048 threads be resident (its loop needs fewer; the reduction at
+// its end would otherwise take two or four more and cost a quarter of the
+// CTAs).  Every other kernel takes the registers it wants (K loaded vectors
+// must stay in registers).
 template <int K, int CTA, int DT>
 constexpr int ldg_min_blocks() {
-    return (DT == SL_BF16 && K <= 8 && CTA >= 256) ? 1024 / CTA : 1;
+    if (DT == SL_BF16) return K <= 8 && CTA >= 256 ? 1024 / CTA : 1;
+    return K == 1 ? 2048 / CTA : 1;
 }
 
 // ---- coverage audit ------------------------------------------------------------
@@ -314,11 +318,14 @@ __device__ __forceinline__ void cta_finish(const Acc<DT>& acc, bool folds, uint3
                                            const KArgs& a, const uint32_t* cta_err = nullptr) {
     __shared__ WarpPartial sp[32];
     const uint32_t lane = threadIdx.x & 31;
-    // A launch that may have started before the previous one finished
-    // (programmatic dependent launch) touches the shared scratch (partials,
+    // A pass that started streaming before the previous launch finished
+    // (a.overlap) touches the shared scratch (partials,
     // window, CTA counter) only once that launch has completed and its writes
     // are visible; without a prerequisite grid this returns at once.
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    // From here on the next launch on the stream may start: its CTAs become
+    // resident, and wait, while this launch's last CTAs reduce.
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (folds) {
         uint32_t s = acc.s;
         uint64_t x = (static_cast<uint64_t>(acc.xh) << 32) | acc.xl, n = acc.n;
@@ -398,14 +405,20 @@ struct TileCursor {
     }
 };
 
-// Start of a streaming kernel: thread 0 keeps this CTA's %globaltimer start
-// in shared memory (no register holds it through the kernel), and the CTA
-// lets a programmatically dependent next launch begin (griddepcontrol; a
-// no-op unless the next launch asked for programmatic stream serialization).
-// Nothing here touches the launch's scratch: that waits for cta_finish.
-__device__ __forceinline__ void cta_start(const KArgs&) {
+// Start of a streaming kernel.  An ordinary pass waits until the kernel before
+// it on the stream has completed and its writes are visible
+// (griddepcontrol.wait; returns at once unless the launch is a programmatic
+// dependent one); cta_finish later lets the next launch on the stream begin.
+// In that order, so that a dependent launch never starts before everything
+// ahead of this one is complete, as if this launch had been an ordinary one.
+// A pass with a.overlap set (sl_enqueue_steps, whose buffers are only read)
+// lets the next launch begin and streams at once, and waits in cta_finish.
+// Thread 0 keeps this CTA's %globaltimer start in shared memory (no register
+// holds it through the kernel).  Nothing here touches the launch's scratch.
+__device__ __forceinline__ void cta_start(const KArgs& a) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.eq.s32 p, %0, 0;\n\t@p griddepcontrol.wait;\n\t"
+                 "@!p griddepcontrol.launch_dependents;\n\t}" ::"r"(a.overlap) : "memory");
     if (threadIdx.x == 0) cta_start_stamp() = gtimer();
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 }  // namespace sl
