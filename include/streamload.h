@@ -85,7 +85,7 @@ typedef enum { SL_LDG = 0, SL_CPASYNC = 1, SL_TMA = 2, SL_LDSTS = 3, SL_LDG4 = 4
 /* Traversal of the buffer by the CTAs.  SL_ASC / SL_DESC: CTA b takes tiles
  * b, b+grid, ... from the first (or last) tile on (the paper's layout).
  * SL_DYN (SL_LDG, SL_LDG32 and SL_CPASYNC): CTAs claim contiguous chunks of
- * about 1 MiB from an atomic counter; integer results are exact, float sums
+ * whole tiles (a sixth of a CTA's share, at most 128 KiB to 1 MiB) from an atomic counter; integer results are exact, float sums
  * meet the same bound but are not bit-reproducible between runs. */
 typedef enum { SL_ASC = 0, SL_DESC = 1, SL_DYN = 2 } sl_order;
 /* LDG load flavour: SL_COP_CG is the paper's primary cell (ld.global.cg,

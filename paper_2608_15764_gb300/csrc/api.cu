@@ -40,7 +40,8 @@ constexpr uint64_t HOST_CHUNK = 256ull << 20;     // sl_run_host staging chunk
 constexpr uint64_t TIMEOUT_NS = 2000000000ull;     // per-wait bound, normal runs
 constexpr uint64_t DEBUG_TIMEOUT_NS = 50000000ull;  // per-wait bound, fault-injection runs
 constexpr int64_t MAX_GRID = 1 << 20;
-constexpr uint64_t DYN_CHUNK_VEC = 65536;          // SL_DYN chunk: 1 MiB of 16-byte vectors
+constexpr uint64_t DYN_CHUNK = 128ull << 10;       // SL_DYN chunk: bytes a CTA claims at a time, at most,
+constexpr uint64_t DYN_CHUNK_FEW = 1ull << 20;     // ... and where claims are dear or would overrun their counter
 constexpr int32_t STEP_COUNTERS = 4096;            // sl_enqueue_steps: SL_DYN passes per counter segment
 
 thread_local char g_err[1024] = "";
@@ -223,6 +224,28 @@ int copies_per_group(const sl_config* cfg) { return cfg->copies == 0 ? 1 : cfg->
 // CTAs per SM (measured: 4 KiB stages read by 128 or 256 threads).
 int tma_batch(const sl_config* cfg) { return cfg->stage_bytes / 16 >= 4 * cfg->cta ? 4 : 1; }
 
+// Tiles in one SL_DYN chunk, for `tiles` tiles of tile_bytes over all passes
+// dealt to `grid` CTAs.
+//
+// Every CTA should get several claims, or the launch ends on a few CTAs
+// streaming their last chunk alone: 256 MiB in 1 MiB chunks left most of 608
+// CTAs idle (32-byte loads: 57.5 us against 43.6 in 32 KiB chunks; 48 MiB by
+// cp.async 2 x 8, 90.9 us against 16.3).  Six claims per CTA measured best over
+// 8 MiB - 1 GiB (4 to 8 within 3%; 2 or 16 up to 10% slower).  Above that the
+// chunk is 128 KiB, not more: 4 GiB at K = 4, 512 threads takes 570.9 us
+// against 572.9 with 256 KiB and 578.0 with 1 MiB chunks, and 564.1 against
+// 566.9 us per overlapped pass.  A claim costs a CTA barrier, which shows where
+// few CTAs share an SM, so a chunk also has 16 tiles per 1, 2, ... CTAs on an
+// SM, up to 1 MiB (FP8 at K = 12, one CTA of 512 threads per SM: 603 us with
+// 1 MiB chunks, 608 with 384 KiB; bfloat16 by cp.async 2 x 8, two CTAs per SM:
+// 576 us per overlapped pass with 512 KiB, 587 with 128 KiB).
+uint64_t dyn_chunk_tiles(uint64_t tiles, uint64_t tile_bytes, uint64_t grid, uint64_t sms) {
+    const uint64_t per_sm = std::max<uint64_t>(1, grid / sms);
+    const uint64_t few = std::max<uint64_t>(1, DYN_CHUNK_FEW / tile_bytes);
+    const uint64_t most = std::min(few, std::max(16 / per_sm, DYN_CHUNK / tile_bytes));
+    return std::min(std::max<uint64_t>(1, tiles / (6 * grid)), std::max<uint64_t>(1, most));
+}
+
 int make_plan(DevCtx* c, const void* buf, uint64_t bytes, int32_t dtype, const sl_config* cfg, Plan* p) {
     if (!cfg) return fail(SL_ERR_ARG, "cfg is NULL");
     if (dtype < SL_U32 || dtype > SL_FP8_E4M3) return fail(SL_ERR_ARG, "bad dtype %d", dtype);
@@ -276,7 +299,6 @@ int make_plan(DevCtx* c, const void* buf, uint64_t bytes, int32_t dtype, const s
         p->block = cta;
         p->smem = 0;
         tile_vec = static_cast<uint64_t>(cta) * cfg->k;
-        if (dyn) tile_vec *= std::max<uint64_t>(1, DYN_CHUNK_VEC / tile_vec);  // chunk of ~1 MiB
         p->warps = cta / 32;
         break;
     case SL_LDG4:
@@ -302,7 +324,6 @@ int make_plan(DevCtx* c, const void* buf, uint64_t bytes, int32_t dtype, const s
         p->block = cta;
         p->smem = 0;
         tile_vec = static_cast<uint64_t>(cta) * cfg->k;  // in 32-byte units
-        if (dyn) tile_vec *= std::max<uint64_t>(1, (DYN_CHUNK_VEC / 2) / tile_vec);
         p->warps = cta / 32;
         break;
     case SL_CPASYNC:
@@ -327,7 +348,6 @@ int make_plan(DevCtx* c, const void* buf, uint64_t bytes, int32_t dtype, const s
         p->smem = static_cast<size_t>(cfg->k) * g * cta * 16 +
                   (((cfg->debug_flags >> SL_DEBUG_SMEM_SKEW_SHIFT) & 7) ? 128 : 0);  // room for a skewed ring
         tile_vec = static_cast<uint64_t>(cta) * cfg->k * g;
-        if (dyn) tile_vec *= std::max<uint64_t>(1, DYN_CHUNK_VEC / tile_vec);  // chunk of ~1 MiB
         p->warps = cta / 32;
         break;
     }
@@ -401,11 +421,22 @@ int make_plan(DevCtx* c, const void* buf, uint64_t bytes, int32_t dtype, const s
     // fixed-iteration control: iters tiles per CTA, all grid*iters tiles wrap
     // around the buffer; otherwise the tiles that cover the buffer once
     const uint64_t fixed_iters = fixed ? cfg->target_loads / (static_cast<uint64_t>(grid) * tile_vec) : 0;
-    const uint64_t ntiles = fixed ? fixed_iters * static_cast<uint64_t>(grid) : (units + tile_vec - 1) / tile_vec;
+    uint64_t ntiles = fixed ? fixed_iters * static_cast<uint64_t>(grid) : (units + tile_vec - 1) / tile_vec;
+    uint64_t total = ntiles * passes;
+    if (dyn) {  // a "tile" of the plan is a chunk: whole tiles, claimed at once
+        const uint64_t tile = tile_vec, tile_bytes = tile * (cfg->mech == SL_LDG32 ? 32 : 16);
+        const uint64_t few = std::max<uint64_t>(1, DYN_CHUNK_FEW / tile_bytes);
+        for (uint64_t n : {dyn_chunk_tiles(total, tile_bytes, static_cast<uint64_t>(grid),
+                                            static_cast<uint64_t>(c->info.sm_count)), few}) {
+            tile_vec = tile * n;
+            ntiles = (units + tile_vec - 1) / tile_vec;
+            total = ntiles * passes;
+            if (total + 3 * static_cast<uint64_t>(grid) < (1ull << 32)) break;
+        }
+    }
     p->grid = (nvec == 0 || (fixed && fixed_iters == 0)) ? 0 : grid;
     // The kernels count tiles and per-thread loads in 32 bits (the per-warp
     // TMA ring's chunk index runs up to total + stages * grid).
-    const uint64_t total = ntiles * passes;
     const uint64_t per_thread = ((total + grid - 1) / grid) * ((tile_vec + cta - 1) / cta);
     // (SL_DYN counters run up to three claims per CTA past the last chunk)
     const uint64_t ahead = static_cast<uint64_t>(grid) *
@@ -417,7 +448,7 @@ int make_plan(DevCtx* c, const void* buf, uint64_t bytes, int32_t dtype, const s
     a.buf = buf;
     a.nvec = nvec;
     a.ntiles = ntiles;
-    a.total = ntiles * passes;
+    a.total = total;
     a.tile_vec = static_cast<uint32_t>(tile_vec);
     a.desc = cfg->order == SL_DESC ? 1 : 0;
     a.next = nullptr;  // set by the caller for SL_DYN

@@ -3,7 +3,7 @@
 // The copies, commit groups and slot ring are those of k_cpasync (D groups of
 // G 16-byte copies per thread in flight, a thread reading back only its own
 // slots), but the CTAs claim contiguous chunks of a.tile_vec vectors (a
-// multiple of the tile cta*D*G, about 1 MiB) from the counter *a.next, as the
+// multiple of the tile cta*D*G) from the counter *a.next, as the
 // dynamic-chunk LDG kernel does, and walk a chunk's tiles in order.  The
 // group refills that run ahead of the fold cross from the last tile of a
 // chunk into the first tile of the next one, so a CTA holds two claims: the
@@ -25,7 +25,6 @@ __global__ void __launch_bounds__(D * G > 8 ? 512 : 1024) k_cpasync_dyn(const KA
     const uint4* __restrict__ buf = static_cast<const uint4*>(a.buf);
     const uint32_t tile = cta * (D * G);
     const uint32_t chunk_vec = a.tile_vec;  // a multiple of tile
-    const uint32_t nchunks = static_cast<uint32_t>(a.ntiles);
     const uint32_t total = static_cast<uint32_t>(a.total);
     const uint64_t nvec = a.nvec;
     const uint32_t skew = (static_cast<uint32_t>(a.debug) >> SL_DEBUG_SMEM_SKEW_SHIFT) & 7u;
@@ -38,7 +37,7 @@ __global__ void __launch_bounds__(D * G > 8 ? 512 : 1024) k_cpasync_dyn(const KA
             len = 0;
             return;
         }
-        const uint64_t base = static_cast<uint64_t>(c % nchunks) * chunk_vec;
+        const uint64_t base = dyn_chunk(a, c);
         const uint64_t left = nvec - base;
         len = left < chunk_vec ? static_cast<uint32_t>(left) : chunk_vec;
         p = buf + base + threadIdx.x;
@@ -46,16 +45,11 @@ __global__ void __launch_bounds__(D * G > 8 ? 512 : 1024) k_cpasync_dyn(const KA
     Acc<DT> acc;
     uint32_t full_tiles = 0;
     volatile uint32_t* vs = slot;
-    if (threadIdx.x == 0) {
-        vs[0] = atomicAdd(a.next, 1u);
-        vs[1] = atomicAdd(a.next, 1u);
-    }
-    __syncthreads();
+    if (threadIdx.x == 0) vs[1] = dyn_claim(a);  // on its way during the prologue
     const uint4* cp;  // this thread's first copy in the current chunk
     const uint4* np;  // ... in the next chunk
     uint32_t clen, nlen;
-    chunk(vs[0], cp, clen);
-    chunk(vs[1], np, nlen);
+    chunk(dyn_first(), cp, clen);
     if (clen) {
         // prologue: the D groups of the chunk's first tile
 #pragma unroll
@@ -71,9 +65,11 @@ __global__ void __launch_bounds__(D * G > 8 ? 512 : 1024) k_cpasync_dyn(const KA
             cp_async_commit();
         }
     }
+    __syncthreads();
+    chunk(vs[1], np, nlen);
 #pragma unroll 1
     for (uint32_t it = 0; clen; ++it) {
-        if (threadIdx.x == 0) vs[(it + 2) % 3] = atomicAdd(a.next, 1u);
+        if (threadIdx.x == 0) vs[(it + 2) % 3] = dyn_claim(a);
         const uint32_t ntl = (clen + tile - 1) / tile;
 #pragma unroll 1
         for (uint32_t t = 0; t < ntl; ++t) {

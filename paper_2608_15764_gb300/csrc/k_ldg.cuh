@@ -76,8 +76,9 @@ __global__ void __launch_bounds__(CTA, ldg_min_blocks<K, CTA, DT>()) k_ldg(const
 }
 
 // SL_DYN traversal: CTAs claim contiguous chunks of a.tile_vec vectors (a
-// multiple of CTA*K, about 1 MiB) from the counter *a.next, so each CTA
-// streams long contiguous runs and faster CTAs take more chunks.  Within a
+// multiple of CTA*K, sized by the host: dyn_chunk_tiles) from the counter
+// *a.next, so each CTA streams contiguous runs and faster CTAs take more
+// chunks.  Within a
 // chunk the tiles and loads are those of k_ldg (K independent 16-byte loads
 // per thread per tile, guarded ragged tail).  Thread 0 claims the following
 // chunk while the CTA works on the current one (one CTA barrier per chunk).
@@ -91,18 +92,15 @@ __global__ void __launch_bounds__(CTA, ldg_min_blocks<K, CTA, DT>()) k_ldg_dyn(c
     cta_start(a);
     const uint4* __restrict__ buf = static_cast<const uint4*>(a.buf);
     const uint32_t chunk_vec = a.tile_vec;
-    const uint32_t nchunks = static_cast<uint32_t>(a.ntiles);
     const uint32_t total = static_cast<uint32_t>(a.total);
     Acc<DT> acc;
     uint32_t full_iters = 0;
     volatile uint32_t* vslot = slot;
-    if (threadIdx.x == 0) vslot[0] = atomicAdd(a.next, 1u);
-    __syncthreads();
-    uint32_t cur = vslot[0];
+    uint32_t cur = dyn_first();
 #pragma unroll 1
     for (uint32_t j = 0; cur < total; ++j) {
-        if (threadIdx.x == 0) vslot[(j + 1) & 1] = atomicAdd(a.next, 1u);
-        const uint64_t base = static_cast<uint64_t>(cur % nchunks) * chunk_vec;
+        if (threadIdx.x == 0) vslot[(j + 1) & 1] = dyn_claim(a);
+        const uint64_t base = dyn_chunk(a, cur);
         const uint64_t left = a.nvec - base;
         const uint32_t len = left < chunk_vec ? static_cast<uint32_t>(left) : chunk_vec;
         const uint4* p = buf + base + threadIdx.x;

@@ -11,7 +11,7 @@
 // 16-byte vectors has a half unit at the end: the thread whose unit index is
 // the first past the whole units loads that last 16-byte vector instead.
 // The grid-stride kernel walks tiles like k_ldg; the SL_DYN kernel claims
-// ~1 MiB chunks like k_ldg_dyn.  issued_loads counts loads: 32-byte loads plus
+// chunks like k_ldg_dyn.  issued_loads counts loads: 32-byte loads plus
 // the one 16-byte load of a half unit, per pass.
 #include "sl_device.cuh"
 
@@ -110,18 +110,14 @@ __global__ void __launch_bounds__(CTA, K == 1 ? 1280 / CTA : 1) k_ldg32_dyn(cons
     const bool half = a.nvec & 1;
     const uint64_t units = n32 + (half ? 1 : 0);
     const uint32_t chunk = a.tile_vec;
-    const uint32_t nchunks = static_cast<uint32_t>(a.ntiles);
     const uint32_t total = static_cast<uint32_t>(a.total);
     Acc<DT> acc;
-    uint32_t full_iters = 0;
     volatile uint32_t* vslot = slot;
-    if (threadIdx.x == 0) vslot[0] = atomicAdd(a.next, 1u);
-    __syncthreads();
-    uint32_t cur = vslot[0];
+    uint32_t cur = dyn_first();
 #pragma unroll 1
     for (uint32_t j = 0; cur < total; ++j) {
-        if (threadIdx.x == 0) vslot[(j + 1) & 1] = atomicAdd(a.next, 1u);
-        const uint64_t base = static_cast<uint64_t>(cur % nchunks) * chunk;
+        if (threadIdx.x == 0) vslot[(j + 1) & 1] = dyn_claim(a);
+        const uint64_t base = dyn_chunk(a, cur);
         const uint64_t left = units - base;
         const uint32_t len = left < chunk ? static_cast<uint32_t>(left) : chunk;
         // whole tiles of whole units only: a chunk holding the half unit ends
@@ -146,13 +142,12 @@ __global__ void __launch_bounds__(CTA, K == 1 ? 1280 / CTA : 1) k_ldg32_dyn(cons
                 acc.fold(v[k].hi);
             }
         }
-        full_iters += nfull;
+        acc.n += nfull * K;
         if (nfull * TILE < len)
             ragged32<K, CTA, DT, COV>(a, buf, base + static_cast<uint64_t>(nfull) * TILE, n32, half, acc);
         __syncthreads();  // the prefetched claim is visible; the slot read next is not rewritten until j+2
         cur = vslot[(j + 1) & 1];
     }
-    acc.n += full_iters * K;
     cta_finish<DT>(acc, true, threadIdx.x >> 5, CTA / 32, a);
 }
 

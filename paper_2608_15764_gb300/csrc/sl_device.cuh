@@ -405,6 +405,24 @@ struct TileCursor {
     }
 };
 
+// SL_DYN: first unit of the chunk that claim c stands for.
+__device__ __forceinline__ uint64_t dyn_chunk(const KArgs& a, uint32_t c) {
+    const uint32_t nchunks = static_cast<uint32_t>(a.ntiles);
+    if (c >= nchunks) c %= nchunks;  // a later pass
+    return static_cast<uint64_t>(c) * a.tile_vec;
+}
+
+// SL_DYN: a CTA's first claim is its own index, so that it starts without a
+// round trip to the counter; the counter deals the rest.  (Read by hand: with
+// blockIdx.x the compiler treats the first chunk apart from the others and some
+// kernels take a few registers more.)
+__device__ __forceinline__ uint32_t dyn_first() {
+    uint32_t c;
+    asm volatile("mov.u32 %0, %%ctaid.x;" : "=r"(c));
+    return c;
+}
+__device__ __forceinline__ uint32_t dyn_claim(const KArgs& a) { return gridDim.x + atomicAdd(a.next, 1u); }
+
 // Start of a streaming kernel.  An ordinary pass waits until the kernel before
 // it on the stream has completed and its writes are visible
 // (griddepcontrol.wait; returns at once unless the launch is a programmatic
