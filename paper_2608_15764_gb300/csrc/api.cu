@@ -394,8 +394,9 @@ int make_plan(DevCtx* c, const void* buf, uint64_t bytes, int32_t dtype, const s
     // registers below that (CTA 1024 with large K), the compiler interleaves
     // loads with folds and K would no longer be the offered ILP.
     // (the fixed-iteration kernel keeps fewer values live besides the loaded
-    // vectors: its floor is K vectors + pointer, tile start and checksum)
-    if ((cfg->mech == SL_LDG || cfg->mech == SL_LDSTS) && fi->regs < 4 * cfg->k + (fixed ? 8 : 16))
+    // vectors: its floor is K vectors + pointer, tile start and checksum: 55
+    // registers at K = 12)
+    if ((cfg->mech == SL_LDG || cfg->mech == SL_LDSTS) && fi->regs < 4 * cfg->k + (fixed ? 7 : 16))
         return fail(SL_ERR_INFEASIBLE, "%d registers per thread cannot hold K=%d loads in flight at cta %d",
                     fi->regs, cfg->k, cta);
     if (cfg->mech == SL_LDG32 && fi->regs < 8 * cfg->k + 16)
@@ -452,6 +453,9 @@ int make_plan(DevCtx* c, const void* buf, uint64_t bytes, int32_t dtype, const s
     a.tile_vec = static_cast<uint32_t>(tile_vec);
     a.desc = cfg->order == SL_DESC ? 1 : 0;
     a.next = nullptr;  // set by the caller for SL_DYN
+    // CTAs with at least one tile (the per-warp TMA ring deals tiles to warps)
+    const uint64_t per_cta = cfg->mech == SL_TMA && cfg->tma_ring == SL_RING_WARP ? cta / 32 : 1;
+    a.active = static_cast<uint32_t>(std::min<uint64_t>(grid, (total + per_cta - 1) / per_cta));
     a.nst = cfg->mech == SL_TMA ? cfg->stages : 0;
     a.debug = cfg->debug_flags;
     a.timeout_ns = (cfg->debug_flags & SL_DEBUG_TMA_SKIP_STAGE) ? DEBUG_TIMEOUT_NS : TIMEOUT_NS;
@@ -984,6 +988,7 @@ int sl_run_host(const void* host_buf, uint64_t bytes, int32_t dtype, const sl_co
         a.window = sl::ctrl_window(c->err);
         a.err = c->err;
         a.result = nullptr;  // combined over all chunks below
+        a.active = static_cast<uint32_t>(p.grid);  // every CTA writes its partial
         a.done = nullptr;
         if (cfg->order == SL_DYN) {  // no last-CTA reset here: clear the chunk counter per launch
             a.next = sl::ctrl_next(c->err);

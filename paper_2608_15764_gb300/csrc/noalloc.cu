@@ -178,6 +178,7 @@ extern "C" int sl_run_noalloc(const void* dev_buf, uint64_t bytes, int32_t dtype
         a.timeout_ns = 2000000000ull;
         a.result = dev_out;  // the last CTA writes the result
         a.done = sl::ctrl_done(ctrl);
+        a.active = static_cast<uint32_t>(a.total < grid ? a.total : grid);
         void* args[] = {&a};
         if (cudaLaunchKernel(fn, dim3(static_cast<unsigned>(grid)), dim3(cta), args, 0, s) != cudaSuccess) {
             (void)cudaGetLastError();

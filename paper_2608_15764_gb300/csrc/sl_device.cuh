@@ -201,17 +201,36 @@ __device__ __forceinline__ void Acc<DT>::float_part(float& hi, float& lo) const 
     df_add(hi, lo, f2_lane1(fs), f2_lane1(fe));
 }
 
-// Shuffle-butterfly reduction of one partial per lane: every lane ends with
-// the warp total (integer parts exact; float pairs combined as double-float
-// with TwoSum, in the butterfly's fixed order).
+// ---- warp reductions ------------------------------------------------------------
+// Integer parts go through the warp-reduce instructions (redux.sync: one
+// instruction per 32-bit word, where a shuffle butterfly is five dependent
+// shuffles and adds); double-float pairs go through shuffles.
+__device__ __forceinline__ uint32_t warp_add32(uint32_t v) { return __reduce_add_sync(FULL_MASK, v); }
+__device__ __forceinline__ uint64_t warp_xor64(uint64_t v) {
+    const uint32_t lo = __reduce_xor_sync(FULL_MASK, static_cast<uint32_t>(v));
+    const uint32_t hi = __reduce_xor_sync(FULL_MASK, static_cast<uint32_t>(v >> 32));
+    return (static_cast<uint64_t>(hi) << 32) | lo;
+}
+// Exact 64-bit sum (mod 2^64) of one value per lane: three pieces of 22, 22
+// and 20 bits, each of whose 32-lane sums fits 32 bits.
+__device__ __forceinline__ uint64_t warp_add64(uint64_t v) {
+    const uint32_t p0 = __reduce_add_sync(FULL_MASK, static_cast<uint32_t>(v) & 0x3FFFFFu);
+    const uint32_t p1 = __reduce_add_sync(FULL_MASK, static_cast<uint32_t>(v >> 22) & 0x3FFFFFu);
+    const uint32_t p2 = __reduce_add_sync(FULL_MASK, static_cast<uint32_t>(v >> 44));
+    return static_cast<uint64_t>(p0) + (static_cast<uint64_t>(p1) << 22) + (static_cast<uint64_t>(p2) << 44);
+}
+
+// Reduction of one partial per lane: every lane ends with the warp total
+// (integer parts exact; float pairs combined as double-float with TwoSum, in
+// the butterfly's fixed order).
 template <int DT>
 __device__ __forceinline__ void warp_merge(uint32_t& s, uint64_t& x, uint64_t& n, float& hi, float& lo) {
+    s = warp_add32(s);
+    x = warp_xor64(x);
+    n = warp_add64(n);
+    if constexpr (DT != SL_U32) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        s += __shfl_xor_sync(FULL_MASK, s, o);
-        x ^= __shfl_xor_sync(FULL_MASK, x, o);
-        n += __shfl_xor_sync(FULL_MASK, n, o);
-        if constexpr (DT != SL_U32) {
+        for (int o = 16; o > 0; o >>= 1) {
             const float ohi = __shfl_xor_sync(FULL_MASK, hi, o);
             const float olo = __shfl_xor_sync(FULL_MASK, lo, o);
             df_add(hi, lo, ohi, olo);
@@ -219,23 +238,22 @@ __device__ __forceinline__ void warp_merge(uint32_t& s, uint64_t& x, uint64_t& n
     }
 }
 
-// Final combine of all CTAs' partials into one sl_result, run by the whole
-// CTA that finished last: thread t folds partials t, t+blockDim, ... in index
-// order (FP64 for the float part: (double)hi + (double)lo), then the warps
-// and the per-warp results are merged by fixed shuffle butterflies, so the
-// float sum has a fixed order for a given launch shape.  Integer parts are
-// exact.  The device error word becomes the status and is cleared; the CTA
-// counter, the chunk counter (if any) and the timing window are reset for the
-// next launch.
-template <typename T, typename Op>
-__device__ __forceinline__ T warp_all(T v, Op op) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = op(v, __shfl_xor_sync(FULL_MASK, v, o));
-    return v;
-}
-
-// Loops are not unrolled and each field is reduced on its own, so that this
-// code needs fewer registers than the streaming loop it follows.
+// Final combine of the partials of all CTAs that took part into one sl_result,
+// run by the whole CTA that finished last: thread t folds partials t,
+// t+blockDim, ... in index order (FP64 for the float part: (double)hi +
+// (double)lo), then the warps and the per-warp results are merged in a fixed
+// order, so the float sum has a fixed order for a given launch shape.  Integer
+// parts are exact.  The device error word becomes the status and is cleared;
+// the CTA counter, the chunk counter (if any) and the timing window are reset
+// for the next launch.
+//
+// This is a chain of L2 round trips at the end of every launch, so what can
+// overlap does: the window and the error word are copied to shared memory
+// while the partials are read (0.4-0.5 us of every launch), and the integer
+// fields are reduced by redux.sync (0.1-0.6 us, most where many warps finish
+// at once).  Loops are not unrolled and each field is reduced on its own, so
+// that this code needs fewer registers than the streaming loop it follows: one
+// more than 32 in the leanest kernels would cost a quarter of their CTAs.
 __device__ __forceinline__ void final_combine(const KArgs& a) {
     struct Fin {
         uint32_t sum;
@@ -244,7 +262,14 @@ __device__ __forceinline__ void final_combine(const KArgs& a) {
     };
     __shared__ Fin fw[32];
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-    const uint32_t n = gridDim.x;
+    const uint32_t n = a.active;
+    // the window and the error word (with its 16 bytes) are copied to shared
+    // memory while the partials are read: no register holds them
+    __shared__ __align__(16) uint64_t swin[2];
+    __shared__ __align__(16) uint32_t serr[4];
+    if (threadIdx.x == blockDim.x - 1)
+        asm volatile("cp.async.cg.shared.global [%0], [%2], 16;\n\tcp.async.cg.shared.global [%1], [%3], 16;"
+                     ::"r"(smem_addr(swin)), "r"(smem_addr(serr)), "l"(a.window), "l"(a.err) : "memory");
     Fin v{0u, 0ull, 0ull, 0.0};
 #pragma unroll 1
     for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) {
@@ -255,17 +280,15 @@ __device__ __forceinline__ void final_combine(const KArgs& a) {
         v.n += (static_cast<uint64_t>(hi4.y) << 32) | hi4.x;
         v.f += static_cast<double>(__uint_as_float(hi4.z)) + static_cast<double>(__uint_as_float(hi4.w));
     }
-    const auto add32 = [](uint32_t p, uint32_t q) { return p + q; };
-    const auto add64 = [](uint64_t p, uint64_t q) { return p + q; };
-    const auto xor64 = [](uint64_t p, uint64_t q) { return p ^ q; };
-    const auto addf = [](double p, double q) { return p + q; };
     for (int pass = 0; pass < 2; ++pass) {  // pass 0: within warps; pass 1: across warps (warp 0)
-        v.sum = warp_all(v.sum, add32);
-        v.x = warp_all(v.x, xor64);
-        v.n = warp_all(v.n, add64);
-        v.f = warp_all(v.f, addf);
+        v.sum = warp_add32(v.sum);
+        v.x = warp_xor64(v.x);
+        v.n = warp_add64(v.n);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v.f += __shfl_xor_sync(FULL_MASK, v.f, o);
         if (pass == 1) break;
         if (lane == 0) fw[warp] = v;
+        asm volatile("cp.async.wait_all;" ::: "memory");
         __syncthreads();
         if (warp != 0) return;
         v = lane < nw ? fw[lane] : Fin{0u, 0ull, 0ull, 0.0};
@@ -277,15 +300,14 @@ __device__ __forceinline__ void final_combine(const KArgs& a) {
         r->xor_u64 = v.x;
         r->issued_loads = v.n;
         r->device_ns = 0;
-        volatile uint64_t* w = a.window;
-        const uint64_t t0 = w[0], t1 = w[1];
+        const uint64_t t0 = swin[0], t1 = swin[1];
         r->window_ns = t1 > t0 ? t1 - t0 : 0;
         r->fsum = v.f;
         const float hi = static_cast<float>(v.f);
         r->fsum_hi = hi;
         r->fsum_lo = static_cast<float>(v.f - static_cast<double>(hi));
         r->sum_u32 = v.sum;
-        r->status = *reinterpret_cast<volatile uint32_t*>(a.err) ? SL_ERR_TIMEOUT : SL_OK;
+        r->status = serr[0] ? SL_ERR_TIMEOUT : SL_OK;
         r->grid = 0;
         r->cta = 0;
         r->resident_per_sm = 0;
@@ -293,8 +315,8 @@ __device__ __forceinline__ void final_combine(const KArgs& a) {
         *a.err = 0;
         *a.done = 0;
         if (a.next) *a.next = 0;
-        w[0] = ~0ull;
-        w[1] = 0;
+        a.window[0] = ~0ull;
+        a.window[1] = 0;
     }
 }
 
@@ -310,7 +332,8 @@ __device__ __forceinline__ uint64_t& cta_start_stamp() {
 // after a CTA barrier warp 0 merges the warp partials (butterfly, fixed
 // order) into the CTA's partial a.parts[blockIdx.x], and thread 0 raises the
 // launch's end stamp to this CTA's %globaltimer.  With
-// a.result set, the last CTA to get here then runs final_combine.  `fw` is
+// a.result set, the last of the a.active CTAs to get here then runs
+// final_combine.  `fw` is
 // this warp's index among the nfw (<= 32) folding warps; `cta_err`, if given,
 // is a CTA-local error code (shared memory) that thread 0 publishes to *a.err.
 template <int DT>
@@ -377,7 +400,7 @@ __device__ __forceinline__ void cta_finish(const Acc<DT>& acc, bool folds, uint3
     __shared__ int s_last;
     if (threadIdx.x == 0) {
         __threadfence();
-        s_last = (atomicAdd(a.done, 1u) == gridDim.x - 1);
+        s_last = (atomicAdd(a.done, 1u) == a.active - 1);
     }
     __syncthreads();
     if (s_last) {
@@ -431,11 +454,19 @@ __device__ __forceinline__ uint32_t dyn_claim(const KArgs& a) { return gridDim.x
 // ahead of this one is complete, as if this launch had been an ordinary one.
 // A pass with a.overlap set (sl_enqueue_steps, whose buffers are only read)
 // lets the next launch begin and streams at once, and waits in cta_finish.
-// Thread 0 keeps this CTA's %globaltimer start in shared memory (no register
-// holds it through the kernel).  Nothing here touches the launch's scratch.
+// A CTA that the launch has no tile for (index a.active or more) exits at once,
+// so that a small launch does not wait for hundreds of empty partials (64 KiB,
+// 8 CTAs of 608 with work: 6.2 -> 4.7 us).  Thread 0 keeps this CTA's
+// %globaltimer start in shared memory (no register holds it through the
+// kernel).  Nothing here touches the launch's scratch.
 __device__ __forceinline__ void cta_start(const KArgs& a) {
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.eq.s32 p, %0, 0;\n\t@p griddepcontrol.wait;\n\t"
-                 "@!p griddepcontrol.launch_dependents;\n\t}" ::"r"(a.overlap) : "memory");
+    asm volatile("{\n\t.reg .pred p;\n\t.reg .u32 b;\n\t"
+                 "mov.u32 b, %%ctaid.x;\n\t"
+                 "setp.ge.u32 p, b, %1;\n\t"
+                 "@p exit;\n\t"
+                 "setp.eq.s32 p, %0, 0;\n\t"
+                 "@p griddepcontrol.wait;\n\t"
+                 "@!p griddepcontrol.launch_dependents;\n\t}" ::"r"(a.overlap), "r"(a.active) : "memory");
     if (threadIdx.x == 0) cta_start_stamp() = gtimer();
 }
 

@@ -45,6 +45,10 @@ struct KArgs {
                             // partials into *result (else a separate combine)
     uint32_t* done;         // CTAs finished (zero before the launch; the last
                             // CTA resets it)
+    uint32_t active;        // CTAs 0 .. active-1 take part in the launch; the
+                            // others have no tile and exit at once (the grid
+                            // itself where result is NULL: a separate combine
+                            // reads every CTA's partial)
     uint32_t* next;         // SL_DYN traversal: next chunk to claim (zero before
                             // the launch; the last CTA resets it), else NULL
     uint32_t* cov;          // coverage instantiations only: one counter per
