@@ -423,13 +423,14 @@ typedef struct sl_batch sl_batch;  /* opaque */
  * persistent kernel per size class streaming many uneven buffers, in one
  * CUDA-graph launch; no paper counterpart).  Each buffer goes to the first
  * table entry that matches it (SL_ERR_ARG if none).  Buffers are cut into
- * work items of at most 1 MiB; each class kernel runs a persistent grid whose
+ * work items (a part of a CTA's share of its class, at most 256 KiB; TMA
+ * classes 128 KiB to 1 MiB); each class kernel runs a persistent grid whose
  * CTAs claim items from an atomic counter, fold them with the class's
- * mechanism and write one partial per warp per item; a combine kernel with
- * one warp per buffer adds each buffer's partials (integer parts exactly,
- * float parts in FP64, in a fixed order) into its sl_result.  The graph --
- * a memset of the counters, the class kernels as parallel branches, then the
- * combine -- is captured once here and replayed by sl_batch_run.  The batch
+ * mechanism and write the item's partials (one; TMA classes one per warp); a
+ * combine kernel with one CTA per buffer adds each buffer's partials (integer
+ * parts exactly, float parts in FP64, in a fixed order) into its sl_result.
+ * The graph -- the class kernels as parallel branches, then the combine -- is
+ * captured once here and replayed by sl_batch_run.  The batch
  * owns its device tables, results, streams and graph until sl_batch_destroy;
  * the caller keeps the buffers alive and unchanged in size.  Asynchronous
  * work of other calls must not overlap a batch run on the same buffers'

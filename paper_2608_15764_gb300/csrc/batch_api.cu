@@ -3,11 +3,11 @@
 // Planning: each buffer goes to the first tuning-table entry that matches
 // its dtype and size; buffers of one entry (a size class) and one dtype form
 // a group that one persistent class kernel streams.  Buffers are cut into
-// work items of at most ITEM_BYTES; each item owns one partial slot per
-// folding warp of its group's kernel, and a buffer's items (hence its slots)
-// are contiguous.  The CUDA graph -- memset of the item counters and the
-// error word, the class kernels as parallel branches, then the per-buffer
-// combine -- is captured once and replayed by sl_batch_run.
+// work items (item_bytes); each item owns the partial slots its kernel writes
+// for it, and a buffer's items (hence its slots) are contiguous.  The CUDA
+// graph -- the class kernels as parallel branches, then the per-buffer combine,
+// which writes the results to page-locked host memory -- is captured once and
+// replayed by sl_batch_run.
 #include <algorithm>
 #include <cstring>
 #include <map>
@@ -20,8 +20,9 @@ namespace sl {
 const void* batch_ldg_kernel(int dtype, int k, int cta);
 const void* batch_cpasync_kernel(int dtype, int d);
 const void* batch_tma_kernel(int dtype, int batch);
-cudaError_t launch_batch_combine(const BufSeg* segs, uint32_t nbuf, const WarpPartial* parts, const uint32_t* err,
-                                 sl_result* out, cudaStream_t s);
+cudaError_t launch_batch_combine(const BufSeg* segs, uint32_t nbuf, const WarpPartial* parts, uint32_t* err,
+                                 uint32_t* next, uint32_t nclasses, sl_result* out, uint32_t* host_err,
+                                 cudaStream_t s);
 }  // namespace sl
 
 namespace {
@@ -30,7 +31,6 @@ using sl::BatchItem;
 using sl::BufSeg;
 using sl::WarpPartial;
 
-constexpr uint64_t ITEM_BYTES = 1ull << 20;
 constexpr uint64_t TIMEOUT_NS = 2000000000ull;
 
 int bfail(int code, const char* msg) { return sl::set_error(code, msg); }
@@ -51,10 +51,14 @@ struct Group {
     const void* fn = nullptr;
     int block = 0;
     size_t smem = 0;
-    int grid = 0;
-    uint32_t warps = 0;       // folding warps per CTA (partial slots per item)
+    int ctas = 0;             // persistent CTAs (resident per SM x SMs, or the entry's grid)
+    int grid = 0;             // ... that the class has items for
+    uint32_t slots = 0;       // partial slots per item
+    uint64_t unit = 0;        // bytes an item is a multiple of (but for a buffer's last one)
+    uint64_t bytes = 0;       // of all its buffers
     std::vector<BatchItem> items;
     uint64_t item_off = 0;    // offset of this group's items in the device item array
+    uint64_t part_off = 0;    // offset of this group's partials
 };
 
 }  // namespace
@@ -67,11 +71,9 @@ struct sl_batch {
     BatchItem* d_items = nullptr;
     BufSeg* d_segs = nullptr;
     WarpPartial* d_parts = nullptr;
-    sl_result* d_results = nullptr;
     uint32_t* d_ctrl = nullptr;  // [0]: error word; [16 + g]: item counter of group g
-    size_t ctrl_bytes = 0;
-    sl_result* h_results = nullptr;
-    uint32_t* h_err = nullptr;   // pinned copy of the error word after each run
+    sl_result* h_results = nullptr;  // page-locked, written by the combine kernel
+    uint32_t* h_err = nullptr;   // page-locked copy of the error word after each run
     cudaStream_t stream = nullptr;
     std::vector<cudaStream_t> branch;
     std::vector<cudaEvent_t> branch_ev;
@@ -95,7 +97,6 @@ void release(sl_batch* b) {
     cudaFree(b->d_items);
     cudaFree(b->d_segs);
     cudaFree(b->d_parts);
-    cudaFree(b->d_results);
     cudaFree(b->d_ctrl);
     cudaFreeHost(b->h_results);
     cudaFreeHost(b->h_err);
@@ -117,14 +118,16 @@ int plan_group(Group& g, int sms, int smem_optin) {
         if (!g.fn) return bfail(SL_ERR_ARG, "tuning entry: no batched LDG kernel (K in {1,2,3,4,6,8,12,16}, cta 128/256/512)");
         g.block = c.cta;
         g.smem = 0;
-        g.warps = c.cta / 32;
+        g.slots = 1;
+        g.unit = static_cast<uint64_t>(c.k) * c.cta * 16;
         break;
     case SL_CPASYNC:
         g.fn = sl::batch_cpasync_kernel(g.dtype, c.k);
         if (!g.fn) return bfail(SL_ERR_ARG, "tuning entry: cp.async depth not in 1..8");
         g.block = c.cta;
         g.smem = static_cast<size_t>(c.k) * c.cta * 16;
-        g.warps = c.cta / 32;
+        g.slots = 1;
+        g.unit = static_cast<uint64_t>(c.k) * c.cta * 16;
         break;
     case SL_TMA:
         if (c.stage_bytes != 4096 && c.stage_bytes != 16384 && c.stage_bytes != 65536)
@@ -139,7 +142,8 @@ int plan_group(Group& g, int sms, int smem_optin) {
         g.fn = sl::batch_tma_kernel(g.dtype, c.stage_bytes / 16 >= 4 * c.cta ? 4 : 1);
         g.block = c.cta + 32;
         g.smem = static_cast<size_t>(c.stages) * c.stage_bytes;
-        g.warps = c.cta / 32;
+        g.slots = c.cta / 32;
+        g.unit = static_cast<uint64_t>(c.stage_bytes);
         break;
     default:
         return bfail(SL_ERR_ARG, "tuning entry: bad mech");
@@ -155,8 +159,29 @@ int plan_group(Group& g, int sms, int smem_optin) {
     int res = 0;
     B_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&res, g.fn, g.block, g.smem), "occupancy query failed");
     if (res < 1) return bfail(SL_ERR_INFEASIBLE, "tuning entry: zero occupancy");
-    g.grid = c.grid > 0 ? c.grid : res * sms;
+    g.ctas = c.grid > 0 ? c.grid : res * sms;
     return SL_OK;
+}
+
+// Bytes of a group's work items, a multiple of its unit (a tile, a ring of
+// cp.async chunks, or a TMA stage).
+//
+// A CTA should get a few items, or a class ends on a few CTAs streaming alone:
+// in 1 MiB items 64 buffers of 16 MiB in all took 66 us on the device, since one
+// CTA needs 44-74 us for a MiB, against 19 in items of a quarter of a CTA's share
+// (three to six items per CTA measure alike, twelve 15% slower).  The TMA class
+// streams on from item to item without draining its ring, but its warps write a
+// partial each at the end of every item: an item is a CTA's share there, at
+// least 128 KiB (64 buffers, 1 GiB, four types: 243 us in items of a sixth of the
+// share, 190 so) and at most 1 MiB (16 GiB of bfloat16: 2,558 us, 2,610 in
+// 256 KiB items).  256 KiB is enough for the others.
+constexpr uint64_t ITEM_MAX = 256ull << 10, ITEM_TMA_MIN = 128ull << 10, ITEM_TMA_MAX = 1ull << 20;
+
+uint64_t item_bytes(const Group& g) {
+    const bool tma = g.cfg.mech == SL_TMA;
+    const uint64_t share = g.bytes / ((tma ? 1 : 4) * static_cast<uint64_t>(g.ctas));
+    const uint64_t want = tma ? std::min(std::max(share, ITEM_TMA_MIN), ITEM_TMA_MAX) : std::min(share, ITEM_MAX);
+    return g.unit * std::max<uint64_t>(1, want / g.unit);
 }
 
 // Everything after the argument checks; the caller releases b on failure.
@@ -188,51 +213,61 @@ int build_batch(sl_batch* b, const sl_batch_desc* descs, int32_t n, const sl_tun
             b->groups.push_back(std::move(g));
         }
         b->class_of[i] = gidx[key];
+        b->groups[gidx[key]].bytes += d.bytes;
     }
 
-    // ---- items, partial slots, per-buffer segments (buffers in order)
-    std::vector<BufSeg> segs(n);
-    uint64_t slots = 0;
+    // ---- items (buffers in order), then every group's place in the item and
+    // partial arrays, then each buffer's partial slots
+    std::vector<uint64_t> first(n);  // index of the buffer's first item in its group
     for (int32_t i = 0; i < n; ++i) {
         Group& g = b->groups[b->class_of[i]];
-        segs[i].pstart = static_cast<uint32_t>(slots);
-        const uint64_t bytes = descs[i].bytes;
+        first[i] = g.items.size();
+        const uint64_t bytes = descs[i].bytes, step = item_bytes(g);
         const uint8_t* p = static_cast<const uint8_t*>(descs[i].ptr);
-        for (uint64_t off = 0; off < bytes; off += ITEM_BYTES) {
-            const uint64_t len = std::min<uint64_t>(ITEM_BYTES, bytes - off);
+        for (uint64_t off = 0; off < bytes; off += step) {
             BatchItem it;
             it.ptr = reinterpret_cast<const uint4*>(p + off);
-            it.nvec = static_cast<uint32_t>(len / 16);
-            it.part = static_cast<uint32_t>(slots);
+            it.nvec = static_cast<uint32_t>(std::min(step, bytes - off) / 16);
+            it.pad = 0;
             g.items.push_back(it);
-            slots += g.warps;
         }
-        segs[i].pcount = static_cast<uint32_t>(slots - segs[i].pstart);
-        if (slots >= (1ull << 32)) return bfail(SL_ERR_ARG, "batch too large");
     }
     std::vector<BatchItem> all;
+    uint64_t slots = 0;
     for (Group& g : b->groups) {
         g.item_off = all.size();
+        g.part_off = slots;
         all.insert(all.end(), g.items.begin(), g.items.end());
+        slots += g.items.size() * g.slots;
+        g.grid = static_cast<int>(std::min<uint64_t>(g.ctas, g.items.size()));
+    }
+    // (the kernels count items, claims past the last one included, and slots in 32 bits)
+    if (slots >= (1ull << 31)) return bfail(SL_ERR_ARG, "batch too large");
+    std::vector<BufSeg> segs(n);
+    for (int32_t i = 0; i < n; ++i) {
+        const Group& g = b->groups[b->class_of[i]];
+        const uint64_t step = item_bytes(g);
+        segs[i].pstart = static_cast<uint32_t>(g.part_off + first[i] * g.slots);
+        segs[i].pcount = static_cast<uint32_t>((descs[i].bytes + step - 1) / step * g.slots);
     }
 
     // ---- device tables (allocated before capture)
     const size_t ng = b->groups.size();
-    b->ctrl_bytes = (16 + ng) * sizeof(uint32_t);
+    const size_t ctrl_bytes = (16 + ng) * sizeof(uint32_t);
     B_TRY(cudaMalloc(&b->d_items, std::max<size_t>(all.size(), 1) * sizeof(BatchItem)), "cudaMalloc failed");
     B_TRY(cudaMalloc(&b->d_segs, std::max<size_t>(n, 1) * sizeof(BufSeg)), "cudaMalloc failed");
     B_TRY(cudaMalloc(&b->d_parts, std::max<uint64_t>(slots, 1) * sizeof(WarpPartial)), "cudaMalloc failed");
-    B_TRY(cudaMalloc(&b->d_results, std::max<size_t>(n, 1) * sizeof(sl_result)), "cudaMalloc failed");
-    B_TRY(cudaMalloc(&b->d_ctrl, b->ctrl_bytes), "cudaMalloc failed");
+    B_TRY(cudaMalloc(&b->d_ctrl, ctrl_bytes), "cudaMalloc failed");
     B_TRY(cudaMallocHost(&b->h_results, std::max<size_t>(n, 1) * sizeof(sl_result)), "cudaMallocHost failed");
     B_TRY(cudaMallocHost(&b->h_err, sizeof(uint32_t)), "cudaMallocHost failed");
     if (!all.empty())
         B_TRY(cudaMemcpy(b->d_items, all.data(), all.size() * sizeof(BatchItem), cudaMemcpyHostToDevice), "copy failed");
     if (n > 0) B_TRY(cudaMemcpy(b->d_segs, segs.data(), n * sizeof(BufSeg), cudaMemcpyHostToDevice), "copy failed");
-    B_TRY(cudaMemset(b->d_ctrl, 0, b->ctrl_bytes), "memset failed");
+    *b->h_err = 0;
 
     // ---- streams and events, then capture the graph
     B_TRY(cudaStreamCreateWithFlags(&b->stream, cudaStreamNonBlocking), "stream create failed");
+    B_TRY(cudaMemsetAsync(b->d_ctrl, 0, ctrl_bytes, b->stream), "memset failed");  // every run leaves it so
     B_TRY(cudaEventCreate(&b->e0), "event create failed");
     B_TRY(cudaEventCreate(&b->e1), "event create failed");
     B_TRY(cudaEventCreateWithFlags(&b->fork_ev, cudaEventDisableTiming), "event create failed");
@@ -245,8 +280,7 @@ int build_batch(sl_batch* b, const sl_batch_desc* descs, int32_t n, const sl_tun
         b->branch_ev.push_back(e);
     }
     B_TRY(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal), "begin capture failed");
-    cudaError_t ce = cudaMemsetAsync(b->d_ctrl, 0, b->ctrl_bytes, b->stream);
-    if (ce == cudaSuccess) ce = cudaEventRecord(b->fork_ev, b->stream);
+    cudaError_t ce = cudaEventRecord(b->fork_ev, b->stream);
     for (size_t g = 0; g < ng && ce == cudaSuccess; ++g) {
         Group& gr = b->groups[g];
         ce = cudaStreamWaitEvent(b->branch[g], b->fork_ev, 0);
@@ -256,7 +290,7 @@ int build_batch(sl_batch* b, const sl_batch_desc* descs, int32_t n, const sl_tun
         a.nitems = static_cast<uint32_t>(gr.items.size());
         a.stage_bytes = static_cast<uint32_t>(gr.cfg.stage_bytes);
         a.next = b->d_ctrl + 16 + g;
-        a.parts = b->d_parts;
+        a.parts = b->d_parts + gr.part_off;
         a.err = b->d_ctrl;
         a.timeout_ns = TIMEOUT_NS;
         a.nst = gr.cfg.mech == SL_TMA ? gr.cfg.stages : 0;
@@ -266,8 +300,8 @@ int build_batch(sl_batch* b, const sl_batch_desc* descs, int32_t n, const sl_tun
         if (ce == cudaSuccess) ce = cudaStreamWaitEvent(b->stream, b->branch_ev[g], 0);
     }
     if (ce == cudaSuccess)
-        ce = sl::launch_batch_combine(b->d_segs, static_cast<uint32_t>(n), b->d_parts, b->d_ctrl, b->d_results,
-                                      b->stream);
+        ce = sl::launch_batch_combine(b->d_segs, static_cast<uint32_t>(n), b->d_parts, b->d_ctrl, b->d_ctrl + 16,
+                                      static_cast<uint32_t>(ng), b->h_results, b->h_err, b->stream);
     cudaGraph_t graph = nullptr;
     const cudaError_t ee = cudaStreamEndCapture(b->stream, &graph);
     b->graph = graph;
@@ -315,20 +349,15 @@ int sl_batch_run(sl_batch* b, sl_result* per_buffer, uint64_t* total_ns) {
     B_TRY(cudaEventRecord(b->e0, b->stream), "event record failed");
     B_TRY(cudaGraphLaunch(b->exec, b->stream), "graph launch failed");
     B_TRY(cudaEventRecord(b->e1, b->stream), "event record failed");
-    if (per_buffer && b->n > 0)
-        B_TRY(cudaMemcpyAsync(b->h_results, b->d_results, b->n * sizeof(sl_result), cudaMemcpyDeviceToHost, b->stream),
-              "result copy failed");
-    B_TRY(cudaMemcpyAsync(b->h_err, b->d_ctrl, sizeof(uint32_t), cudaMemcpyDeviceToHost, b->stream),
-          "error-word copy failed");
     B_TRY(cudaStreamSynchronize(b->stream), "batch run failed");
     float ms = 0.0f;
     B_TRY(cudaEventElapsedTime(&ms, b->e0, b->e1), "event timing failed");
     if (total_ns) *total_ns = static_cast<uint64_t>(static_cast<double>(ms) * 1e6 + 0.5);
-    int st = *b->h_err ? SL_ERR_TIMEOUT : SL_OK;
+    const int st = *b->h_err ? SL_ERR_TIMEOUT : SL_OK;
     if (per_buffer && b->n > 0) {
         std::memcpy(per_buffer, b->h_results, b->n * sizeof(sl_result));
-        for (int i = 0; i < b->n; ++i)
-            if (per_buffer[i].status != SL_OK) st = per_buffer[i].status;
+        if (st != SL_OK)
+            for (int i = 0; i < b->n; ++i) per_buffer[i].status = st;
     }
     if (st != SL_OK) return bfail(st, "a bounded device wait timed out");
     return SL_OK;

@@ -1,68 +1,133 @@
 // k_batch.cuh -- persistent kernels of the batched form.
 //
-// A batch is cut into work items (a piece of at most 1 MiB of one buffer).
-// Every class kernel runs a persistent grid; its CTAs claim the class's
-// items one at a time from an atomic counter (dynamic balancing across
-// uneven buffers), fold each item with the class's mechanism and write one
-// partial per folding warp per item, at the item's own partial slots, so the
-// result does not depend on which CTA took which item.  kb_combine then adds
-// the partials of each buffer in slot order.
+// A batch is cut into work items (contiguous pieces of one buffer, sized by
+// the host: see item_bytes in batch_api.cu).  Every class kernel runs a
+// persistent grid; CTA b starts on the class's items b and grid + b and claims
+// the others one at a time from an atomic counter (dynamic balancing across
+// uneven buffers), folds each item with the class's mechanism and writes its
+// partials at the item's own slots, so the result does not depend on which CTA
+// took which item.  kb_combine then adds the partials of each buffer in slot
+// order, writes its result straight into page-locked host memory and leaves
+// the counters at zero for the next run: a run is the class kernels and this
+// one, with no memset before them and no copies after them.
 #pragma once
 
 #include "sl_device.cuh"
 
 namespace sl {
 
-struct BatchItem {
+struct __align__(16) BatchItem {
     const uint4* ptr;  // first vector of the item
     uint32_t nvec;     // 16-byte vectors in the item (> 0)
-    uint32_t part;     // first partial slot of the item (one per folding warp)
+    uint32_t pad;
 };
 static_assert(sizeof(BatchItem) == 16, "BatchItem layout");
 
 struct BufSeg {
     uint32_t pstart;  // first partial slot of the buffer
-    uint32_t pcount;  // partial slots of the buffer (items x folding warps)
+    uint32_t pcount;  // partial slots of the buffer (items x slots per item)
 };
 
 struct BArgs {
     const BatchItem* items;  // this class's items
     uint32_t nitems;
     uint32_t stage_bytes;    // TMA stage size
-    uint32_t* next;          // item counter (zeroed before every launch)
-    WarpPartial* parts;      // the batch's partial array
+    uint32_t* next;          // item counter (zero before every launch)
+    WarpPartial* parts;      // this class's partials, in item order
     uint32_t* err;           // device error word
     uint64_t timeout_ns;     // bound of any single device wait (TMA)
     int32_t nst;             // TMA stages
     int32_t reserved;
 };
 
-// Thread 0 claims the next item; every thread of the CTA gets its index.
-__device__ __forceinline__ uint32_t claim_item(const BArgs& a, volatile uint32_t* slot) {
-    if (threadIdx.x == 0) *slot = atomicAdd(a.next, 1u);
-    __syncthreads();
-    const uint32_t i = *slot;
-    __syncthreads();  // everyone has read the slot before it is overwritten
-    return i;
-}
-
-// Reduce a warp's accumulators and let lane 0 write the warp's item partial.
+// Reduce a warp's accumulators into one partial (lane 0 holds it afterwards).
 template <int DT>
-__device__ __forceinline__ void warp_item_store(const Acc<DT>& acc, WarpPartial* dst) {
+__device__ __forceinline__ WarpPartial warp_partial(const Acc<DT>& acc) {
     uint32_t s = acc.s;
     uint64_t x = (static_cast<uint64_t>(acc.xh) << 32) | acc.xl, n = acc.n;
     float hi = 0.0f, lo = 0.0f;
     if constexpr (DT != SL_U32) acc.float_part(hi, lo);
     warp_merge<DT>(s, x, n, hi, lo);
-    if ((threadIdx.x & 31) == 0) {
-        WarpPartial p;
-        p.sum = s;
-        p.pad = 0;
-        p.xr = x;
-        p.issued = n;
-        p.hi = hi;
-        p.lo = lo;
-        *dst = p;
+    WarpPartial p;
+    p.sum = s;
+    p.pad = 0;
+    p.xr = x;
+    p.issued = n;
+    p.hi = hi;
+    p.lo = lo;
+    return p;
+}
+
+// The item loop of a class kernel whose CTAs work on one item together.
+// stream(item, acc) folds an item.  The next item's descriptor is copied to
+// shared memory, and the one after it claimed, while the current item streams;
+// one CTA barrier per item publishes both together with the warps' partials,
+// which one warp (a different one for each item) then merges into the item's
+// partial while the others go on.  (Claiming, fetching the descriptor and two
+// barriers between items left every CTA idle for about 2 us per item.)  Little is kept in registers across stream():
+// the item's index and its place in the loop are re-read from shared memory.
+template <int DT, typename Stream>
+__device__ __forceinline__ void batch_items(const BArgs& a, Stream stream) {
+    __shared__ BatchItem slot[2];
+    __shared__ uint32_t sidx[3];
+    __shared__ WarpPartial wp[2][32];
+    volatile uint32_t* vidx = sidx;
+    if (threadIdx.x == 0) {
+        vidx[0] = blockIdx.x;  // the host launches at most nitems CTAs
+        vidx[1] = blockIdx.x + gridDim.x;
+    }
+    BatchItem it = a.items[dyn_first()];
+#pragma unroll 1
+    for (uint32_t j = 0;; ++j) {
+        // sidx[j % 3]: this item, [(j + 1) % 3]: the next, [(j + 2) % 3]: being claimed
+        uint32_t claim = 0xFFFFFFFFu;
+        if (threadIdx.x == 0) {
+            const uint32_t ahead = vidx[(j + 1) % 3];
+            if (ahead < a.nitems) {
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(&slot[(j + 1) & 1])),
+                             "l"(a.items + ahead) : "memory");
+                claim = 2 * gridDim.x + atomicAdd(a.next, 1u);
+            }
+        }
+        {
+            Acc<DT> acc;
+            stream(it, acc);
+            const WarpPartial w = warp_partial<DT>(acc);
+            if ((threadIdx.x & 31) == 0) wp[j & 1][threadIdx.x >> 5] = w;
+        }
+        if (threadIdx.x == 0) {
+            asm volatile("cp.async.wait_all;" ::: "memory");
+            vidx[(j + 2) % 3] = claim;
+        }
+        __syncthreads();
+        const uint32_t cur = vidx[j % 3], next = vidx[(j + 1) % 3];
+        const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+        if (warp == j % nw) {
+            uint32_t s = 0;
+            uint64_t x = 0, n = 0;
+            float hi = 0.0f, lo = 0.0f;
+            if (lane < nw) {
+                const WarpPartial q = wp[j & 1][lane];
+                s = q.sum;
+                x = q.xr;
+                n = q.issued;
+                hi = q.hi;
+                lo = q.lo;
+            }
+            warp_merge<DT>(s, x, n, hi, lo);
+            if (lane == 0) {
+                WarpPartial q;
+                q.sum = s;
+                q.pad = 0;
+                q.xr = x;
+                q.issued = n;
+                q.hi = hi;
+                q.lo = lo;
+                a.parts[cur] = q;
+            }
+        }
+        if (next >= a.nitems) break;
+        it = slot[(j + 1) & 1];
     }
 }
 
@@ -70,14 +135,9 @@ __device__ __forceinline__ void warp_item_store(const Acc<DT>& acc, WarpPartial*
 // loads per thread per tile (same fold and tile layout as k_ldg), guarded
 // ragged tail.
 template <int K, int CTA, int DT>
-__global__ void __launch_bounds__(CTA, ldg_min_blocks<K, CTA, DT>()) kb_ldg(const BArgs a) {
-    __shared__ uint32_t slot;
+__global__ void __launch_bounds__(CTA, DT == SL_BF16 ? ldg_min_blocks<K, CTA, DT>() : 1) kb_ldg(const BArgs a) {
     constexpr uint32_t TILE = static_cast<uint32_t>(CTA) * K;
-    for (;;) {
-        const uint32_t item = claim_item(a, &slot);
-        if (item >= a.nitems) break;
-        const BatchItem it = a.items[item];
-        Acc<DT> acc;
+    batch_items<DT>(a, [](const BatchItem& it, Acc<DT>& acc) {
         const uint32_t nfull = it.nvec / TILE;
         const uint4* p = it.ptr + threadIdx.x;
 #pragma unroll 1
@@ -105,8 +165,7 @@ __global__ void __launch_bounds__(CTA, ldg_min_blocks<K, CTA, DT>()) kb_ldg(cons
                 }
             }
         }
-        warp_item_store<DT>(acc, a.parts + it.part + (threadIdx.x >> 5));
-    }
+    });
 }
 
 }  // namespace sl
