@@ -261,7 +261,7 @@ def sl_batch_run(b: sl_batch, results: bool = True):
     out = (sl_result * max(b.n, 1))() if results else None
     ns = ctypes.c_uint64()
     _check(load().sl_batch_run(b.handle, out, ctypes.byref(ns)))
-    return ([out[i] for i in range(b.n)] if results else None), int(ns.value)
+    return (out[:b.n] if results else None), int(ns.value)
 
 
 def sl_batch_info(b: sl_batch):

@@ -81,8 +81,11 @@ struct DevCtx {
     WarpPartial* parts = nullptr;
     uint64_t parts_cap = 0;
     uint32_t* err = nullptr;    // control block (sl::CTRL_BYTES): error word, CTA counter, window
-    sl_result* dres = nullptr;  // device result of sl_run / sl_run_host
-    sl_result* hres = nullptr;  // pinned host copy
+    sl_result* dres = nullptr;  // device result of sl_chase
+    // page-locked; the kernels of the synchronous calls write [0] in place (a
+    // result copied from device memory took another 5 us of every call), a
+    // sweep's warm-up launch [1]
+    sl_result* hres = nullptr;
     uint64_t* two_dev = nullptr;   // sl_twostream: timer words [0, 8) and results [8, 24)
     uint64_t* two_host = nullptr;  // pinned copy of the results
     uint32_t* step_next = nullptr; // sl_enqueue_steps with SL_DYN: one chunk counter per pass
@@ -146,7 +149,7 @@ int get_ctx(DevCtx** out) {
         CUDA_TRY(cudaMemset(c->err, 0, sl::CTRL_BYTES));
         CUDA_TRY(cudaMemset(sl::ctrl_window(c->err), 0xFF, sizeof(uint64_t)));  // earliest start = ~0
         CUDA_TRY(cudaMalloc(&c->dres, sizeof(sl_result)));
-        CUDA_TRY(cudaMallocHost(&c->hres, sizeof(sl_result)));
+        CUDA_TRY(cudaMallocHost(&c->hres, 2 * sizeof(sl_result)));
         CUDA_TRY(cudaEventCreate(&c->ev0));
         CUDA_TRY(cudaEventCreate(&c->ev1));
         c->flush_bytes = ((2 * static_cast<uint64_t>(c->info.l2_bytes)) + (1u << 20) - 1) & ~((1ull << 20) - 1);
@@ -588,10 +591,9 @@ int enqueue_locked(DevCtx* c, const void* buf, uint64_t bytes, int32_t dtype, co
 int run_locked(DevCtx* c, const void* buf, uint64_t bytes, int32_t dtype, const sl_config* cfg, sl_result* out,
                uint32_t* cov = nullptr) {
     Plan p;
-    int rc = enqueue_locked(c, buf, bytes, dtype, cfg, c->dres, true, &p, cov);
+    int rc = enqueue_locked(c, buf, bytes, dtype, cfg, c->hres, true, &p, cov);
     if (rc) return rc;
     cudaStream_t s = static_cast<cudaStream_t>(cfg->stream);
-    CUDA_TRY(cudaMemcpyAsync(c->hres, c->dres, sizeof(sl_result), cudaMemcpyDeviceToHost, s));
     CUDA_TRY(cudaStreamSynchronize(s));
     float ms = 0.0f;
     CUDA_TRY(cudaEventElapsedTime(&ms, c->ev0, c->ev1));
@@ -772,9 +774,16 @@ int sl_sweep(const void* dev_buf, uint64_t bytes, int32_t dtype, const sl_config
         sl_result* row = out + static_cast<int64_t>(cell) * repeats;
         sl_result tmp;
         int st = SL_OK;
-        for (int32_t w = 0; w < warmup && st == SL_OK; ++w) st = run_locked(c, dev_buf, bytes, dtype, &cells[cell], &tmp);
+        for (int32_t w = 0; w + 1 < warmup && st == SL_OK; ++w)
+            st = run_locked(c, dev_buf, bytes, dtype, &cells[cell], &tmp);
+        // The last warm-up launch is not waited for: the first timed launch
+        // follows it on the stream, and both results are read then.
+        const bool warm = warmup > 0 && st == SL_OK;
+        if (warm) st = enqueue_locked(c, dev_buf, bytes, dtype, &cells[cell], c->hres + 1, false, nullptr);
         for (int32_t r = 0; r < repeats; ++r) {
             if (st == SL_OK) st = run_locked(c, dev_buf, bytes, dtype, &cells[cell], &row[r]);
+            if (warm && r == 0 && st == SL_OK && c->hres[1].status != SL_OK)
+                st = fail(c->hres[1].status, "a bounded device wait timed out");
             if (st != SL_OK) {
                 std::memset(&row[r], 0, sizeof row[r]);
                 row[r].status = st;
@@ -933,9 +942,8 @@ int sl_run_host(const void* host_buf, uint64_t bytes, int32_t dtype, const sl_co
         }
         CUDA_TRY(cudaEventRecord(c->ev0, s));
         Plan p;
-        int rc2 = enqueue_locked(c, dptr, bytes, dtype, cfg, c->dres, false, &p);
+        int rc2 = enqueue_locked(c, dptr, bytes, dtype, cfg, c->hres, false, &p);
         if (rc2) return rc2;
-        CUDA_TRY(cudaMemcpyAsync(c->hres, c->dres, sizeof(sl_result), cudaMemcpyDeviceToHost, s));
         CUDA_TRY(cudaEventRecord(c->ev1, s));
         CUDA_TRY(cudaStreamSynchronize(s));
         float ms = 0.0f;
@@ -1000,8 +1008,7 @@ int sl_run_host(const void* host_buf, uint64_t bytes, int32_t dtype, const sl_co
     }
     if (cfg->order == SL_DYN)  // leave the chunk counter at zero for the next launch
         CUDA_TRY(cudaMemsetAsync(sl::ctrl_next(c->err), 0, sizeof(uint32_t), s));
-    CUDA_TRY(sl::launch_combine(c->parts, per_parts * nchunks, sl::ctrl_window(c->err), c->err, c->dres, s));
-    CUDA_TRY(cudaMemcpyAsync(c->hres, c->dres, sizeof(sl_result), cudaMemcpyDeviceToHost, s));
+    CUDA_TRY(sl::launch_combine(c->parts, per_parts * nchunks, sl::ctrl_window(c->err), c->err, c->hres, s));
     CUDA_TRY(cudaEventRecord(c->ev1, s));
     CUDA_TRY(cudaStreamSynchronize(s));
     float ms = 0.0f;
