@@ -484,30 +484,10 @@ int launch(const Plan& p, cudaStream_t s, LaunchMode mode = LAUNCH_PLAIN) {
     if (p.grid == 0) return SL_OK;
     KArgs a = p.args;
     void* args[] = {&a};
-    if (mode == LAUNCH_WAIT) {
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
-            (void)cudaGetLastError();
-            mode = LAUNCH_PLAIN;
-        }
-    }
-    if (mode == LAUNCH_PLAIN) {
-        CUDA_TRY(cudaLaunchKernel(p.fn, dim3(static_cast<unsigned>(p.grid)), dim3(p.block), args, p.smem, s));
-        return SL_OK;
-    }
-    // may begin once every CTA of the previous kernel on the stream has
-    // executed griddepcontrol.launch_dependents or ended
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t lc{};
-    lc.gridDim = dim3(static_cast<unsigned>(p.grid));
-    lc.blockDim = dim3(p.block);
-    lc.dynamicSmemBytes = p.smem;
-    lc.stream = s;
-    lc.attrs = attr;
-    lc.numAttrs = 1;
-    CUDA_TRY(cudaLaunchKernelExC(&lc, p.fn, args));
+    CUDA_TRY(mode == LAUNCH_PLAIN
+                 ? cudaLaunchKernel(p.fn, dim3(static_cast<unsigned>(p.grid)), dim3(p.block), args, p.smem, s)
+                 : sl::launch_dependent(p.fn, static_cast<unsigned>(p.grid), p.block, p.smem, args, s,
+                                        mode == LAUNCH_OVERLAP));
     return SL_OK;
 }
 
@@ -609,6 +589,28 @@ int run_locked(DevCtx* c, const void* buf, uint64_t bytes, int32_t dtype, const 
 namespace sl {
 // Record a failure for sl_last_error() from another translation unit.
 int set_error(int code, const char* msg) { return fail(code, "%s", msg); }
+
+cudaError_t launch_dependent(const void* fn, unsigned grid, int block, size_t smem, void** args, cudaStream_t s,
+                             bool in_capture) {
+    if (!in_capture) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+            (void)cudaGetLastError();
+            return cudaLaunchKernel(fn, dim3(grid), dim3(block), args, smem, s);
+        }
+    }
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t lc{};
+    lc.gridDim = dim3(grid);
+    lc.blockDim = dim3(block);
+    lc.dynamicSmemBytes = smem;
+    lc.stream = s;
+    lc.attrs = attr;
+    lc.numAttrs = 1;
+    return cudaLaunchKernelExC(&lc, fn, args);
+}
 }  // namespace sl
 
 extern "C" {

@@ -30,6 +30,15 @@ __global__ void __launch_bounds__(256) k_fill_splitmix64(uint4* __restrict__ buf
     }
 }
 
+// The state of a control block before a launch: zero, with the window's
+// earliest start at ~0.  One kernel that the load kernel depends on
+// programmatically: two memset nodes before it cost 4 us more per call.
+__global__ void __launch_bounds__(CTRL_BYTES / 8) k_clear_ctrl(uint64_t* ctrl, uint32_t window) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    ctrl[threadIdx.x] = threadIdx.x == window ? ~0ull : 0ull;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // Overwrite the flush buffer: its lines displace whatever was L2-resident.
 __global__ void __launch_bounds__(256) k_flush(uint4* __restrict__ buf, uint64_t nvec) {
     const uint64_t stride = static_cast<uint64_t>(gridDim.x) * blockDim.x;
@@ -109,6 +118,13 @@ cudaError_t launch_fill_splitmix64(void* buf, uint64_t nvec, uint64_t seed, int 
     if (blocks > cap) blocks = cap;
     k_fill_splitmix64<<<static_cast<unsigned>(blocks), 256, 0, s>>>(static_cast<uint4*>(buf), nvec, seed);
     return cudaGetLastError();
+}
+
+cudaError_t launch_clear_ctrl(void* ctrl, cudaStream_t s) {
+    uint64_t* words = static_cast<uint64_t*>(ctrl);
+    uint32_t window = static_cast<uint32_t>(ctrl_window(ctrl) - words);
+    void* args[] = {&words, &window};
+    return launch_dependent(reinterpret_cast<const void*>(&k_clear_ctrl), 1, CTRL_BYTES / 8, 0, args, s, false);
 }
 
 cudaError_t launch_flush(void* buf, uint64_t nvec, int sms, cudaStream_t s) {

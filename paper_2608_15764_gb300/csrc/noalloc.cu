@@ -155,8 +155,7 @@ extern "C" int sl_run_noalloc(const void* dev_buf, uint64_t bytes, int32_t dtype
     cudaStream_t s = static_cast<cudaStream_t>(cfg->stream);
 
     // error word and CTA counter start at zero, the window at (~0, 0)
-    if (cudaMemsetAsync(ctrl, 0, sl::CTRL_BYTES, s) != cudaSuccess ||
-        cudaMemsetAsync(sl::ctrl_window(ctrl), 0xFF, sizeof(uint64_t), s) != cudaSuccess) {
+    if (sl::launch_clear_ctrl(ctrl, s) != cudaSuccess) {
         (void)cudaGetLastError();
         return na_fail(SL_ERR_CUDA, "clearing the control block failed");
     }
@@ -180,7 +179,11 @@ extern "C" int sl_run_noalloc(const void* dev_buf, uint64_t bytes, int32_t dtype
         a.done = sl::ctrl_done(ctrl);
         a.active = static_cast<uint32_t>(a.total < grid ? a.total : grid);
         void* args[] = {&a};
-        if (cudaLaunchKernel(fn, dim3(static_cast<unsigned>(grid)), dim3(cta), args, 0, s) != cudaSuccess) {
+        // dependent on the clear, but for several passes (as sl_enqueue)
+        const cudaError_t e =
+            passes > 1 ? cudaLaunchKernel(fn, dim3(static_cast<unsigned>(grid)), dim3(cta), args, 0, s)
+                       : sl::launch_dependent(fn, static_cast<unsigned>(grid), cta, 0, args, s, false);
+        if (e != cudaSuccess) {
             (void)cudaGetLastError();
             return na_fail(SL_ERR_CUDA, "kernel launch failed");
         }

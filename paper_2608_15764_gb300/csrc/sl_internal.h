@@ -116,7 +116,16 @@ cudaError_t launch_chase(const uint32_t* chain, uint64_t nwords, uint32_t start,
 // Record a failure message for sl_last_error(); returns code (api.cu).
 int set_error(int code, const char* msg);
 
+// Programmatic dependent launch (api.cu): the kernel may begin once every CTA
+// of the previous kernel on the stream has executed
+// griddepcontrol.launch_dependents or ended.  While the stream is being
+// captured: an ordinary launch, unless in_capture.
+cudaError_t launch_dependent(const void* fn, unsigned grid, int block, size_t smem, void** args, cudaStream_t s,
+                             bool in_capture);
+
 // Utility launches (k_util.cu); asynchronous on `s`.
+// launch_clear_ctrl puts a control block into the state that a launch expects.
+cudaError_t launch_clear_ctrl(void* ctrl, cudaStream_t s);
 cudaError_t launch_fill_splitmix64(void* buf, uint64_t nvec, uint64_t seed, int sms, cudaStream_t s);
 cudaError_t launch_flush(void* buf, uint64_t nvec, int sms, cudaStream_t s);
 cudaError_t launch_combine(const WarpPartial* parts, uint64_t nparts, uint64_t* window, uint32_t* err,

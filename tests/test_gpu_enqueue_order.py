@@ -24,7 +24,7 @@ def sl():
 
 
 def _sums(sl, out, n):
-    return [int(v) & 0xFFFFFFFF for v in out.view(torch.int32).view(n, sl.RESULT_BYTES // 4)[:, 12].cpu()]
+    return [int(v) & 0xFFFFFFFF for v in out[: n * sl.RESULT_BYTES].view(torch.int32).view(n, sl.RESULT_BYTES // 4)[:, 12].cpu()]
 
 
 @pytest.mark.parametrize("mech,kw", POINTS)
@@ -73,3 +73,32 @@ def test_enqueue_under_capture(sl, mech, kw):
             total += i + 1
             want.append((total * (nbytes // 4)) & 0xFFFFFFFF)
         assert _sums(sl, out, n) == want
+
+
+@pytest.mark.parametrize("passes", [1, 2])
+@pytest.mark.parametrize("nbytes", [16, (1 << 20) + 16 * 37])
+def test_noalloc_order_and_capture(sl, nbytes, passes):
+    """sl_run_noalloc clears its control block and reads the buffer in stream
+    order, back to back, between writers, and replayed from a graph."""
+    n = 16
+    buf = torch.zeros(nbytes // 4, dtype=torch.int32, device="cuda")
+    out = torch.zeros(n * sl.RESULT_BYTES, dtype=torch.uint8, device="cuda")
+    cfg = sl.config("ldg", k=2, cta=128, passes=passes)
+    for i in range(n):
+        if i % 2 == 0:
+            buf.fill_(i + 1)
+        sl.sl_run_noalloc(buf, out[i * sl.RESULT_BYTES:], dtype=sl.SL_U32, cfg=cfg)
+    assert _sums(sl, out, n) == [(passes * (i // 2 * 2 + 1) * (nbytes // 4)) & 0xFFFFFFFF for i in range(n)]
+    stream = torch.cuda.Stream()
+    cfg = sl.config("ldg", k=2, cta=128, passes=passes, stream=stream)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=stream):
+        for i in range(2):
+            buf.fill_(i + 7)
+            sl.sl_run_noalloc(buf, out[i * sl.RESULT_BYTES:], dtype=sl.SL_U32, cfg=cfg)
+    for _ in range(3):
+        out.zero_()
+        g.replay()
+        torch.cuda.synchronize()
+        assert _sums(sl, out, 2) == [(passes * (i + 7) * (nbytes // 4)) & 0xFFFFFFFF for i in range(2)]
