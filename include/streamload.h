@@ -306,9 +306,10 @@ int sl_sweep(const void* dev_buf, uint64_t bytes, int32_t dtype, const sl_config
              sl_result* out);
 
 /* End-to-end form: the payload is in HOST memory (page-locked for full
- * speed).  Staged mode (cfg->host_direct == 0): copies it to a library-owned
- * device staging ring in chunks of 256 MiB on a copy stream, overlapped with
- * the load kernel on each chunk, then combines all chunks.  Direct mode
+ * speed).  Staged mode (cfg->host_direct == 0): up to 64 MiB, copies it to a
+ * library-owned device staging buffer in one piece; above, to a staging ring in
+ * chunks of 64 to 256 MiB on a copy stream, overlapped with the load kernel on
+ * each chunk, then combines all chunks.  Direct mode
  * (cfg->host_direct != 0): one load kernel reads the host buffer in place
  * through its device mapping (SL_ERR_ARG if the device cannot address it).
  * Either way the result is copied back and device_ns covers the whole call

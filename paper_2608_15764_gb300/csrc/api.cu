@@ -36,7 +36,8 @@ using sl::KArgs;
 using sl::WarpPartial;
 
 constexpr int MAX_DEVICES = 64;
-constexpr uint64_t HOST_CHUNK = 256ull << 20;     // sl_run_host staging chunk
+constexpr uint64_t HOST_CHUNK = 256ull << 20;     // sl_run_host staging buffer
+constexpr uint64_t HOST_ONE = 64ull << 20;        // ... payloads up to this are not cut
 constexpr uint64_t TIMEOUT_NS = 2000000000ull;     // per-wait bound, normal runs
 constexpr uint64_t DEBUG_TIMEOUT_NS = 50000000ull;  // per-wait bound, fault-injection runs
 constexpr int64_t MAX_GRID = 1 << 20;
@@ -964,12 +965,22 @@ int sl_run_host(const void* host_buf, uint64_t bytes, int32_t dtype, const sl_co
         }
         CUDA_TRY(cudaStreamCreateWithFlags(&c->copy_stream, cudaStreamNonBlocking));
     }
-    const uint64_t chunk = std::min<uint64_t>(bytes, HOST_CHUNK);
-    const uint64_t nchunks = bytes == 0 ? 0 : (bytes + HOST_CHUNK - 1) / HOST_CHUNK;
+    // Up to 64 MiB the payload is copied in one piece on the caller's own stream
+    // and its kernel combines by itself, as sl_run's does: a chunk on the copy
+    // stream costs about 8 us in events between the streams, more than the
+    // kernel it would hide (256 KiB: 36 us by chunks and a combine kernel, 25 so;
+    // 1 MiB: 60 / 35; 64 MiB: 362 / 353, in eight chunks 373).  Above, in four
+    // chunks of at least 64 MiB (128 MiB: 683 us, 691 in eight), so that only the
+    // last one's kernel is not hidden behind the link.
+    const uint64_t step = std::min(HOST_CHUNK, std::max(HOST_ONE, (bytes / 4 + (1u << 20) - 1) >> 20 << 20));
+    const uint64_t chunk = std::min<uint64_t>(bytes, step);
+    const uint64_t nchunks = bytes == 0 ? 0 : (bytes + step - 1) / step;
     // One launch shape for every chunk (planned on a full chunk), so every
-    // chunk's kernel writes all of its partial slots.
+    // chunk's kernel writes all of its partial slots.  What may be launched is
+    // decided for a whole staging buffer, however the payload is cut.
     Plan p;
-    rc = make_plan(c, c->stage[0], chunk, dtype, cfg, &p);
+    rc = make_plan(c, c->stage[0], std::min<uint64_t>(bytes, HOST_CHUNK), dtype, cfg, &p);
+    if (rc == SL_OK) rc = make_plan(c, c->stage[0], chunk, dtype, cfg, &p);
     if (rc) return rc;
     const uint64_t per_parts = static_cast<uint64_t>(p.grid);  // one partial per CTA
     rc = ensure_scratch(c, per_parts * nchunks);
@@ -977,11 +988,19 @@ int sl_run_host(const void* host_buf, uint64_t bytes, int32_t dtype, const sl_co
     const uint64_t passes = cfg->passes == 0 ? 1 : static_cast<uint64_t>(cfg->passes);
 
     CUDA_TRY(cudaEventRecord(c->ev0, s));
-    CUDA_TRY(cudaStreamWaitEvent(c->copy_stream, c->ev0, 0));
-    for (uint64_t i = 0; i < nchunks; ++i) {
+    if (nchunks == 1) {
+        CUDA_TRY(cudaMemcpyAsync(c->stage[0], host_buf, bytes, cudaMemcpyHostToDevice, s));
+        sl_config one = *cfg;
+        one.flush_l2 = 0;  // as for chunks
+        rc = enqueue_locked(c, c->stage[0], bytes, dtype, &one, c->hres, false, &p);
+        if (rc) return rc;
+    } else {
+        CUDA_TRY(cudaStreamWaitEvent(c->copy_stream, c->ev0, 0));
+    }
+    for (uint64_t i = 0; i < nchunks && nchunks > 1; ++i) {
         const int b = static_cast<int>(i & 1);
-        const uint64_t off = i * HOST_CHUNK;
-        const uint64_t len = std::min<uint64_t>(HOST_CHUNK, bytes - off);
+        const uint64_t off = i * step;
+        const uint64_t len = std::min<uint64_t>(step, bytes - off);
         if (i >= 2) CUDA_TRY(cudaStreamWaitEvent(c->copy_stream, c->consumed[b], 0));
         CUDA_TRY(cudaMemcpyAsync(c->stage[b], static_cast<const uint8_t*>(host_buf) + off, len,
                                  cudaMemcpyHostToDevice, c->copy_stream));
@@ -1008,9 +1027,10 @@ int sl_run_host(const void* host_buf, uint64_t bytes, int32_t dtype, const sl_co
         CUDA_TRY(cudaLaunchKernel(p.fn, dim3(static_cast<unsigned>(p.grid)), dim3(p.block), args, p.smem, s));
         CUDA_TRY(cudaEventRecord(c->consumed[b], s));
     }
-    if (cfg->order == SL_DYN)  // leave the chunk counter at zero for the next launch
+    if (cfg->order == SL_DYN && nchunks > 1)  // leave the chunk counter at zero for the next launch
         CUDA_TRY(cudaMemsetAsync(sl::ctrl_next(c->err), 0, sizeof(uint32_t), s));
-    CUDA_TRY(sl::launch_combine(c->parts, per_parts * nchunks, sl::ctrl_window(c->err), c->err, c->hres, s));
+    if (nchunks != 1)
+        CUDA_TRY(sl::launch_combine(c->parts, per_parts * nchunks, sl::ctrl_window(c->err), c->err, c->hres, s));
     CUDA_TRY(cudaEventRecord(c->ev1, s));
     CUDA_TRY(cudaStreamSynchronize(s));
     float ms = 0.0f;

@@ -66,6 +66,7 @@ __global__ void __launch_bounds__(COMBINE_THREADS) k_combine(const WarpPartial* 
     uint32_t sum = 0;
     uint64_t xr = 0, n = 0;
     double f = 0.0;
+#pragma unroll 4
     for (uint64_t i = t; i < nparts; i += COMBINE_THREADS) {
         const WarpPartial p = parts[i];
         sum += p.sum;
