@@ -186,6 +186,7 @@ struct Plan {
     int resident = 0;         // occupancy-API CTAs per SM
     uint64_t warps = 0;       // folding warps per CTA (each CTA writes one partial)
     KArgs args{};
+    uint32_t prefetch = 0;    // KArgs::prefetch of a dependent launch
 };
 
 int func_info(DevCtx* c, const void* fn, size_t smem, FuncInfo** out) {
@@ -248,6 +249,27 @@ uint64_t dyn_chunk_tiles(uint64_t tiles, uint64_t tile_bytes, uint64_t grid, uin
     const uint64_t few = std::max<uint64_t>(1, DYN_CHUNK_FEW / tile_bytes);
     const uint64_t most = std::min(few, std::max(16 / per_sm, DYN_CHUNK / tile_bytes));
     return std::min(std::max<uint64_t>(1, tiles / (6 * grid)), std::max<uint64_t>(1, most));
+}
+
+// Bytes that each CTA of a dependent launch prefetches into L2 (tile_bytes: one
+// tile of the configuration).  Where a CTA starts with 32 KiB or more in flight
+// (cp.async and TMA rings, large tiles) 32 KiB pay: 48 MiB of bfloat16 by
+// cp.async 2 x 8 enqueued back to back 16.0 -> 14.5 us (16 KiB: 15.3), 96 MiB of
+// FP8 by TMA 20.6 -> 19.3, 64 MiB at K = 8 15.5 -> 14.6; dynamic chunks of plain
+// loads take 16 KiB (256 MiB 41.7 -> 41.0, 96 MiB 19.7 -> 19.1; 19.5 with 32).
+// Grid-stride plain loads with small tiles do without: 64 MiB at K = 4 took 15.4
+// us with 16 KiB and 15.1 without, 1 GiB at K = 2 177 and 173.
+uint32_t first_bytes(const sl_config* cfg, uint64_t tile_bytes) {
+    switch (cfg->mech) {
+    case SL_LDG:
+    case SL_LDG32:
+        if (cfg->target_loads) return 0;
+        if (cfg->order == SL_DYN) return 16u << 10;
+        return tile_bytes >= 32u << 10 ? 32u << 10 : 0;
+    case SL_CPASYNC: return static_cast<uint32_t>(std::min<uint64_t>(tile_bytes, 32u << 10));
+    case SL_TMA: return cfg->tma_ring == SL_RING_CTA ? 32u << 10 : 0;
+    default: return 0;
+    }
 }
 
 int make_plan(DevCtx* c, const void* buf, uint64_t bytes, int32_t dtype, const sl_config* cfg, Plan* p) {
@@ -428,8 +450,9 @@ int make_plan(DevCtx* c, const void* buf, uint64_t bytes, int32_t dtype, const s
     const uint64_t fixed_iters = fixed ? cfg->target_loads / (static_cast<uint64_t>(grid) * tile_vec) : 0;
     uint64_t ntiles = fixed ? fixed_iters * static_cast<uint64_t>(grid) : (units + tile_vec - 1) / tile_vec;
     uint64_t total = ntiles * passes;
+    const uint64_t tile_bytes = tile_vec * (cfg->mech == SL_LDG32 ? 32 : cfg->mech == SL_LDG4 ? 4 : 16);
     if (dyn) {  // a "tile" of the plan is a chunk: whole tiles, claimed at once
-        const uint64_t tile = tile_vec, tile_bytes = tile * (cfg->mech == SL_LDG32 ? 32 : 16);
+        const uint64_t tile = tile_vec;
         const uint64_t few = std::max<uint64_t>(1, DYN_CHUNK_FEW / tile_bytes);
         for (uint64_t n : {dyn_chunk_tiles(total, tile_bytes, static_cast<uint64_t>(grid),
                                             static_cast<uint64_t>(c->info.sm_count)), few}) {
@@ -460,6 +483,7 @@ int make_plan(DevCtx* c, const void* buf, uint64_t bytes, int32_t dtype, const s
     // CTAs with at least one tile (the per-warp TMA ring deals tiles to warps)
     const uint64_t per_cta = cfg->mech == SL_TMA && cfg->tma_ring == SL_RING_WARP ? cta / 32 : 1;
     a.active = static_cast<uint32_t>(std::min<uint64_t>(grid, (total + per_cta - 1) / per_cta));
+    p->prefetch = first_bytes(cfg, tile_bytes);
     a.nst = cfg->mech == SL_TMA ? cfg->stages : 0;
     a.debug = cfg->debug_flags;
     a.timeout_ns = (cfg->debug_flags & SL_DEBUG_TMA_SKIP_STAGE) ? DEBUG_TIMEOUT_NS : TIMEOUT_NS;
@@ -484,6 +508,7 @@ enum LaunchMode { LAUNCH_PLAIN, LAUNCH_WAIT, LAUNCH_OVERLAP };
 int launch(const Plan& p, cudaStream_t s, LaunchMode mode = LAUNCH_PLAIN) {
     if (p.grid == 0) return SL_OK;
     KArgs a = p.args;
+    if (mode == LAUNCH_WAIT) a.prefetch = p.prefetch;
     void* args[] = {&a};
     CUDA_TRY(mode == LAUNCH_PLAIN
                  ? cudaLaunchKernel(p.fn, dim3(static_cast<unsigned>(p.grid)), dim3(p.block), args, p.smem, s)

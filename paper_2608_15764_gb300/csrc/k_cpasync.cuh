@@ -33,7 +33,7 @@ __global__ void __launch_bounds__(D * G > 8 ? 512 : 1024) k_cpasync(const KArgs 
     // [D*G][cta]: slot j = k*G + g holds copy j of a tile.  128-byte aligned;
     // an experiment flag (SL_DEBUG_SMEM_SKEW) can shift it by 16-byte steps.
     extern __shared__ __align__(128) uint4 ring[];
-    cta_start(a);
+    cta_start(a, a.tile_vec * 16);
     const uint32_t cta = blockDim.x;
     const uint4* __restrict__ buf = static_cast<const uint4*>(a.buf);
     const uint32_t ntiles = static_cast<uint32_t>(a.ntiles);

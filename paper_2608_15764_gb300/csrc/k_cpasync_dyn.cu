@@ -20,7 +20,7 @@ template <int D, int G, int DT, bool COV = false>
 __global__ void __launch_bounds__(D * G > 8 ? 512 : 1024) k_cpasync_dyn(const KArgs a) {
     extern __shared__ __align__(128) uint4 ring[];
     __shared__ uint32_t slot[3];
-    cta_start(a);
+    cta_start(a, a.tile_vec * 16);
     const uint32_t cta = blockDim.x;
     const uint4* __restrict__ buf = static_cast<const uint4*>(a.buf);
     const uint32_t tile = cta * (D * G);

@@ -25,7 +25,7 @@ __global__ void __launch_bounds__(CTA, ldg_min_blocks<K, CTA, DT>()) k_ldg(const
     // whose kernel would spill are rejected on the host (local memory > 0), as
     // the paper requires zero spills (§3).
     constexpr uint32_t TILE = static_cast<uint32_t>(CTA) * K;
-    cta_start(a);
+    cta_start(a, TILE * 16);
     const uint4* __restrict__ buf = static_cast<const uint4*>(a.buf);
     const uint32_t ntiles = static_cast<uint32_t>(a.ntiles);
     const uint32_t total = static_cast<uint32_t>(a.total);
@@ -89,7 +89,7 @@ template <int K, int CTA, int DT, bool COV = false>
 __global__ void __launch_bounds__(CTA, ldg_min_blocks<K, CTA, DT>()) k_ldg_dyn(const KArgs a) {
     constexpr uint32_t TILE = static_cast<uint32_t>(CTA) * K;
     __shared__ uint32_t slot[2];
-    cta_start(a);
+    cta_start(a, a.tile_vec * 16);
     const uint4* __restrict__ buf = static_cast<const uint4*>(a.buf);
     const uint32_t chunk_vec = a.tile_vec;
     const uint32_t total = static_cast<uint32_t>(a.total);

@@ -57,7 +57,7 @@ __device__ __forceinline__ void ragged32(const KArgs& a, const Oct* buf, uint64_
 template <int K, int CTA, int DT, bool COV = false>
 __global__ void __launch_bounds__(CTA, 1) k_ldg32(const KArgs a) {
     constexpr uint32_t TILE = static_cast<uint32_t>(CTA) * K;
-    cta_start(a);
+    cta_start(a, TILE * 32);
     const Oct* __restrict__ buf = static_cast<const Oct*>(a.buf);
     const uint64_t n32 = a.nvec >> 1;
     const bool half = a.nvec & 1;
@@ -104,7 +104,7 @@ template <int K, int CTA, int DT, bool COV = false>
 __global__ void __launch_bounds__(CTA, K == 1 ? 1280 / CTA : 1) k_ldg32_dyn(const KArgs a) {
     constexpr uint32_t TILE = static_cast<uint32_t>(CTA) * K;
     __shared__ uint32_t slot[2];
-    cta_start(a);
+    cta_start(a, a.tile_vec * 32);
     const Oct* __restrict__ buf = static_cast<const Oct*>(a.buf);
     const uint64_t n32 = a.nvec >> 1;
     const bool half = a.nvec & 1;

@@ -27,7 +27,7 @@ __device__ __forceinline__ uint32_t ldg4(const uint32_t* p) {
 template <int K, int CTA>
 __global__ void __launch_bounds__(CTA, 1) k_ldg4(const KArgs a) {
     constexpr uint32_t TILE = static_cast<uint32_t>(CTA) * K;
-    cta_start(a);
+    cta_start<false>(a);
     const uint32_t* __restrict__ buf = static_cast<const uint32_t*>(a.buf);
     const uint32_t ntiles = static_cast<uint32_t>(a.ntiles);
     const uint32_t total = static_cast<uint32_t>(a.total);

@@ -21,7 +21,7 @@ namespace sl {
 template <int K, int CTA, bool COV = false>
 __global__ void __launch_bounds__(CTA, 1) k_ldg_fixed(const KArgs a) {
     constexpr uint32_t TILE = static_cast<uint32_t>(CTA) * K;
-    cta_start(a);
+    cta_start<false>(a);
     const uint4* __restrict__ buf = static_cast<const uint4*>(a.buf);
     const uint64_t nvec = a.nvec;
     const uint32_t total = static_cast<uint32_t>(a.total);  // iters * grid tiles

@@ -22,7 +22,7 @@ __device__ __forceinline__ void sts16(uint32_t saddr, const uint4& v) {
 template <int G, int DT, bool COV = false>
 __global__ void __launch_bounds__(G <= 8 ? 1024 : 256, 1) k_ldsts(const KArgs a) {
     extern __shared__ __align__(128) uint4 st_ring[];  // [G][cta]; 128-byte aligned (+ SL_DEBUG_SMEM_SKEW)
-    cta_start(a);
+    cta_start<false>(a);
     const uint32_t cta = blockDim.x;
     const uint4* __restrict__ buf = static_cast<const uint4*>(a.buf);
     const uint32_t ntiles = static_cast<uint32_t>(a.ntiles);

@@ -41,7 +41,7 @@ __global__ void __launch_bounds__(1024, 1) k_tma(const KArgs a) {
     __shared__ volatile int abort_flag;
     __shared__ uint32_t cta_err;  // a bounded wait's error code, published to *a.err by cta_finish
 
-    cta_start(a);
+    cta_start(a, a.tile_vec * 16);
     const uint32_t nst = static_cast<uint32_t>(a.nst);
     const uint32_t ntiles = static_cast<uint32_t>(a.ntiles);
     const uint32_t total = static_cast<uint32_t>(a.total);
@@ -177,7 +177,7 @@ __global__ void __launch_bounds__(SL_MAX_STAGES * 32, 4) k_tma_warp(const KArgs 
     __shared__ volatile int abort_flag;
     __shared__ uint32_t cta_err;
 
-    cta_start(a);
+    cta_start<false>(a);
     const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
     const uint32_t nst = static_cast<uint32_t>(a.nst) / nw;  // stages of this warp (the host checks W | stages)
     // chunk indices fit in 32 bits: the host checks total + grid * W < 2^32

@@ -459,14 +459,35 @@ __device__ __forceinline__ uint32_t dyn_claim(const KArgs& a) { return gridDim.x
 // 8 CTAs of 608 with work: 6.2 -> 4.7 us).  Thread 0 keeps this CTA's
 // %globaltimer start in shared memory (no register holds it through the
 // kernel).  Nothing here touches the launch's scratch.
-__device__ __forceinline__ void cta_start(const KArgs& a) {
+//
+// A dependent launch with a.prefetch set first asks L2 for what the CTA will
+// read first, before it waits: its CTAs are resident during the last few
+// microseconds of the kernel before it, when DRAM is nearly idle.  (A prefetch
+// returns no data and L2 is where that kernel's writes go, so the loads after
+// the wait see them.)  tile_bytes: bytes of one of the launch's tiles (chunks
+// for SL_DYN); PF false leaves this out.
+template <bool PF = true>
+__device__ __forceinline__ void cta_start(const KArgs& a, uint32_t tile_bytes = 0) {
     asm volatile("{\n\t.reg .pred p;\n\t.reg .u32 b;\n\t"
                  "mov.u32 b, %%ctaid.x;\n\t"
-                 "setp.ge.u32 p, b, %1;\n\t"
-                 "@p exit;\n\t"
+                 "setp.ge.u32 p, b, %0;\n\t"
+                 "@p exit;\n\t}" ::"r"(a.active) : "memory");
+    if (PF && a.prefetch && threadIdx.x == 0) {
+        const uint32_t ntiles = static_cast<uint32_t>(a.ntiles);
+        const uint32_t part = tile_bytes < a.prefetch ? tile_bytes : a.prefetch;
+        uint32_t it = blockIdx.x;
+        for (uint32_t n = 0; n < a.prefetch && it < ntiles; n += part, it += gridDim.x) {
+            const uint64_t off = static_cast<uint64_t>(a.desc ? ntiles - 1 - it : it) * tile_bytes;
+            const uint64_t left = a.nvec * 16 - off;
+            asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;"
+                         ::"l"(static_cast<const char*>(a.buf) + off), "r"(left < part ? static_cast<uint32_t>(left) : part)
+                         : "memory");
+        }
+    }
+    asm volatile("{\n\t.reg .pred p;\n\t"
                  "setp.eq.s32 p, %0, 0;\n\t"
                  "@p griddepcontrol.wait;\n\t"
-                 "@!p griddepcontrol.launch_dependents;\n\t}" ::"r"(a.overlap), "r"(a.active) : "memory");
+                 "@!p griddepcontrol.launch_dependents;\n\t}" ::"r"(a.overlap) : "memory");
     if (threadIdx.x == 0) cta_start_stamp() = gtimer();
 }
 

@@ -30,6 +30,8 @@ struct KArgs {
     uint32_t tile_vec;      // 16-byte vectors per tile (LDG: cta*K, CPASYNC: cta*D*G,
                             // TMA: stage_bytes/16)
     int32_t desc;           // 1: walk tiles from the last one downward
+    uint32_t prefetch;      // bytes each CTA asks L2 for before it waits for the
+                            // kernel before it (0: none; a multiple of 16)
     int32_t nst;            // TMA: ring stages (per CTA or per warp)
     int32_t debug;          // SL_DEBUG_* flags
     int32_t overlap;        // 1: the launch streams at once and lets the next one
