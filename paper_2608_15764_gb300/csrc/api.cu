@@ -258,8 +258,10 @@ uint64_t dyn_chunk_tiles(uint64_t tiles, uint64_t tile_bytes, uint64_t grid, uin
 // FP8 by TMA 20.6 -> 19.3, 64 MiB at K = 8 15.5 -> 14.6; dynamic chunks of plain
 // loads take 16 KiB (256 MiB 41.7 -> 41.0, 96 MiB 19.7 -> 19.1; 19.5 with 32).
 // Grid-stride plain loads with small tiles do without: 64 MiB at K = 4 took 15.4
-// us with 16 KiB and 15.1 without, 1 GiB at K = 2 177 and 173.
+// us with 16 KiB and 15.1 without, 1 GiB at K = 2 177 and 173.  So do several
+// passes in one launch, which want their CTAs spread evenly (cta_finish).
 uint32_t first_bytes(const sl_config* cfg, uint64_t tile_bytes) {
+    if (cfg->passes > 1) return 0;
     switch (cfg->mech) {
     case SL_LDG:
     case SL_LDG32:
@@ -549,11 +551,6 @@ int enqueue_locked(DevCtx* c, const void* buf, uint64_t bytes, int32_t dtype, co
     int rc = make_plan(c, buf, bytes, dtype, cfg, &p);
     if (rc) return rc;
     cudaStream_t s = static_cast<cudaStream_t>(cfg->stream);
-    // Several passes in one launch: the gap is small beside them, and where the
-    // buffer stays in L2 the SMs' load rate is the bound, which CTAs placed
-    // beside another launch's (not exactly grid / SMs on every SM) would miss:
-    // 16 passes over 32 MiB take 37.0 us as an ordinary launch, 40.6 otherwise.
-    if (mode == LAUNCH_WAIT && cfg->passes > 1) mode = LAUNCH_PLAIN;
     if (cov) {
         // coverage audit: the same launch shape with the counting instantiation
         const void* fn = dtype == SL_U32 ? coverage_fn(cfg) : nullptr;

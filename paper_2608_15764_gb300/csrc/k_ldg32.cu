@@ -99,9 +99,10 @@ __global__ void __launch_bounds__(CTA, 1) k_ldg32(const KArgs a) {
 
 // SL_DYN: chunks of a.tile_vec units claimed from *a.next (the next claim
 // prefetched by thread 0; one CTA barrier per chunk).
-// (K = 1 is held to 48 registers, five 256-thread CTAs per SM.)
+// (K = 1 is held to 32 registers for uint32, 48 for floats: eight and five
+// 256-thread CTAs per SM.)
 template <int K, int CTA, int DT, bool COV = false>
-__global__ void __launch_bounds__(CTA, K == 1 ? 1280 / CTA : 1) k_ldg32_dyn(const KArgs a) {
+__global__ void __launch_bounds__(CTA, K == 1 ? (DT == SL_U32 ? 2048 : 1280) / CTA : 1) k_ldg32_dyn(const KArgs a) {
     constexpr uint32_t TILE = static_cast<uint32_t>(CTA) * K;
     __shared__ uint32_t slot[2];
     cta_start(a, a.tile_vec * 32);

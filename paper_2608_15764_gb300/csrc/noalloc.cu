@@ -179,11 +179,7 @@ extern "C" int sl_run_noalloc(const void* dev_buf, uint64_t bytes, int32_t dtype
         a.done = sl::ctrl_done(ctrl);
         a.active = static_cast<uint32_t>(a.total < grid ? a.total : grid);
         void* args[] = {&a};
-        // dependent on the clear, but for several passes (as sl_enqueue)
-        const cudaError_t e =
-            passes > 1 ? cudaLaunchKernel(fn, dim3(static_cast<unsigned>(grid)), dim3(cta), args, 0, s)
-                       : sl::launch_dependent(fn, static_cast<unsigned>(grid), cta, 0, args, s, false);
-        if (e != cudaSuccess) {
+        if (sl::launch_dependent(fn, static_cast<unsigned>(grid), cta, 0, args, s, false) != cudaSuccess) {
             (void)cudaGetLastError();
             return na_fail(SL_ERR_CUDA, "kernel launch failed");
         }

@@ -345,10 +345,16 @@ __device__ __forceinline__ void cta_finish(const Acc<DT>& acc, bool folds, uint3
     // (a.overlap) touches the shared scratch (partials,
     // window, CTA counter) only once that launch has completed and its writes
     // are visible; without a prerequisite grid this returns at once.
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    // From here on the next launch on the stream may start: its CTAs become
-    // resident, and wait, while this launch's last CTAs reduce.
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    // Where launches prefetch (a.prefetch), the next one on the stream may start
+    // from here on: its CTAs become resident, prefetch and wait while this
+    // launch's last CTAs reduce.  Otherwise it starts as the last CTA exits: its
+    // CTAs then find empty SMs and spread evenly (16 passes over 32 MiB in L2:
+    // 34.6 us, 39.9 where they are placed beside this launch's, 36.9 as an
+    // ordinary launch; 16 MiB 6.35 us against 6.63).
+    asm volatile("{\n\t.reg .pred p;\n\t"
+                 "setp.ne.u32 p, %0, 0;\n\t"
+                 "griddepcontrol.wait;\n\t"
+                 "@p griddepcontrol.launch_dependents;\n\t}" ::"r"(a.prefetch) : "memory");
     if (folds) {
         uint32_t s = acc.s;
         uint64_t x = (static_cast<uint64_t>(acc.xh) << 32) | acc.xl, n = acc.n;
@@ -449,8 +455,8 @@ __device__ __forceinline__ uint32_t dyn_claim(const KArgs& a) { return gridDim.x
 // Start of a streaming kernel.  An ordinary pass waits until the kernel before
 // it on the stream has completed and its writes are visible
 // (griddepcontrol.wait; returns at once unless the launch is a programmatic
-// dependent one); cta_finish later lets the next launch on the stream begin.
-// In that order, so that a dependent launch never starts before everything
+// dependent one); cta_finish, or its end, lets the next launch on the stream
+// begin.  In that order, so that a dependent launch never starts before everything
 // ahead of this one is complete, as if this launch had been an ordinary one.
 // A pass with a.overlap set (sl_enqueue_steps, whose buffers are only read)
 // lets the next launch begin and streams at once, and waits in cta_finish.

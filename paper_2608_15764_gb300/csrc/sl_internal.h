@@ -31,13 +31,13 @@ struct KArgs {
                             // TMA: stage_bytes/16)
     int32_t desc;           // 1: walk tiles from the last one downward
     uint32_t prefetch;      // bytes each CTA asks L2 for before it waits for the
-                            // kernel before it (0: none; a multiple of 16)
+                            // kernel before it (a multiple of 16; 0: none, and
+                            // the next launch does not start before the end)
     int32_t nst;            // TMA: ring stages (per CTA or per warp)
     int32_t debug;          // SL_DEBUG_* flags
     int32_t overlap;        // 1: the launch streams at once and lets the next one
                             // begin (passes over buffers that are only read);
-                            // 0: it waits for the kernel before it first, and
-                            // lets the next one begin as its CTAs finish
+                            // 0: it waits for the kernel before it first
     WarpPartial* parts;     // [grid]: one partial per CTA
     uint64_t* window;       // [2]: earliest CTA start, latest CTA end
                             // (%globaltimer; ~0 and 0 before the launch)
