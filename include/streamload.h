@@ -445,8 +445,9 @@ int sl_batch_create(const sl_batch_desc* descs, int32_t n, const sl_tune_entry* 
  * bounded device wait gave up during the run (with or without per_buffer). */
 int sl_batch_run(sl_batch* b, sl_result* per_buffer, uint64_t* total_ns);
 
-/* Number of class kernels (graph kernel nodes besides the combine) and the
- * class each buffer went to (host array of n, may be NULL). */
+/* Number of classes (tuning entry and dtype; each has a class kernel in the
+ * graph, but small LDG classes of one entry share one) and the class each
+ * buffer went to (host array of n, may be NULL). */
 int sl_batch_info(const sl_batch* b, int32_t* nclasses, int32_t* class_of_buffer);
 
 void sl_batch_destroy(sl_batch* b);

@@ -18,6 +18,7 @@
 
 namespace sl {
 const void* batch_ldg_kernel(int dtype, int k, int cta);
+const void* batch_ldg_any_kernel(int k, int cta);
 const void* batch_cpasync_kernel(int dtype, int d);
 const void* batch_tma_kernel(int dtype, int batch);
 cudaError_t launch_batch_combine(const BufSeg* segs, uint32_t nbuf, const WarpPartial* parts, uint32_t* err,
@@ -52,13 +53,21 @@ struct Group {
     int block = 0;
     size_t smem = 0;
     int ctas = 0;             // persistent CTAs (resident per SM x SMs, or the entry's grid)
-    int grid = 0;             // ... that the class has items for
     uint32_t slots = 0;       // partial slots per item
     uint64_t unit = 0;        // bytes an item is a multiple of (but for a buffer's last one)
     uint64_t bytes = 0;       // of all its buffers
     std::vector<BatchItem> items;
-    uint64_t item_off = 0;    // offset of this group's items in the device item array
     uint64_t part_off = 0;    // offset of this group's partials
+};
+
+// One launch of the graph: a group's class kernel, or several groups of one
+// LDG entry in one kernel for mixed types.
+struct Unit {
+    const void* fn = nullptr;
+    std::vector<int> groups;
+    int ctas = 0;
+    uint64_t nitems = 0;
+    uint64_t item_off = 0, part_off = 0;
 };
 
 }  // namespace
@@ -102,6 +111,22 @@ void release(sl_batch* b) {
     cudaFreeHost(b->h_err);
     (void)cudaGetLastError();
     delete b;
+}
+
+// Persistent CTAs of kernel fn at group g's block shape.
+int plan_ctas(const void* fn, const Group& g, int sms, int* ctas) {
+    cudaFuncAttributes fa;
+    B_TRY(cudaFuncGetAttributes(&fa, fn), "cudaFuncGetAttributes failed");
+    if (fa.localSizeBytes > 0) return bfail(SL_ERR_INFEASIBLE, "tuning entry: kernel spills registers");
+    if (g.block > fa.maxThreadsPerBlock) return bfail(SL_ERR_INFEASIBLE, "tuning entry: too many threads for this kernel");
+    if (g.smem > 0)
+        B_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(g.smem)),
+              "cudaFuncSetAttribute failed");
+    int res = 0;
+    B_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&res, fn, g.block, g.smem), "occupancy query failed");
+    if (res < 1) return bfail(SL_ERR_INFEASIBLE, "tuning entry: zero occupancy");
+    *ctas = g.cfg.grid > 0 ? g.cfg.grid : res * sms;
+    return SL_OK;
 }
 
 // Kernel, block shape, shared memory and persistent grid of one group.
@@ -149,18 +174,7 @@ int plan_group(Group& g, int sms, int smem_optin) {
         return bfail(SL_ERR_ARG, "tuning entry: bad mech");
     }
     if (g.smem > static_cast<size_t>(smem_optin)) return bfail(SL_ERR_INFEASIBLE, "tuning entry: shared memory over the limit");
-    cudaFuncAttributes fa;
-    B_TRY(cudaFuncGetAttributes(&fa, g.fn), "cudaFuncGetAttributes failed");
-    if (fa.localSizeBytes > 0) return bfail(SL_ERR_INFEASIBLE, "tuning entry: kernel spills registers");
-    if (g.block > fa.maxThreadsPerBlock) return bfail(SL_ERR_INFEASIBLE, "tuning entry: too many threads for this kernel");
-    if (g.smem > 0)
-        B_TRY(cudaFuncSetAttribute(g.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(g.smem)),
-              "cudaFuncSetAttribute failed");
-    int res = 0;
-    B_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&res, g.fn, g.block, g.smem), "occupancy query failed");
-    if (res < 1) return bfail(SL_ERR_INFEASIBLE, "tuning entry: zero occupancy");
-    g.ctas = c.grid > 0 ? c.grid : res * sms;
-    return SL_OK;
+    return plan_ctas(g.fn, g, sms, &g.ctas);
 }
 
 // Bytes of a group's work items, a multiple of its unit (a tile, a ring of
@@ -182,6 +196,40 @@ uint64_t item_bytes(const Group& g) {
     const uint64_t share = g.bytes / ((tma ? 1 : 4) * static_cast<uint64_t>(g.ctas));
     const uint64_t want = tma ? std::min(std::max(share, ITEM_TMA_MIN), ITEM_TMA_MAX) : std::min(share, ITEM_MAX);
     return g.unit * std::max<uint64_t>(1, want / g.unit);
+}
+
+// The graph's launches.  The LDG classes that one entry has for several types
+// share a kernel where they have at most two items per CTA: a parallel branch
+// costs the graph about 1.5 us, more than such a class takes, while larger
+// classes want the registers (CTAs per SM) of their own type's kernel.  (64
+// buffers, 16 MiB, four types in two size classes: 19.6 -> 14.0 us on the device,
+// 36 -> 29 per call.)
+int plan_units(const std::vector<Group>& groups, int sms, std::vector<Unit>* units) {
+    std::vector<bool> taken(groups.size(), false);
+    for (size_t i = 0; i < groups.size(); ++i) {
+        if (taken[i] || groups[i].items.empty()) continue;
+        Unit u;
+        if (groups[i].cfg.mech == SL_LDG) {
+            const void* any = sl::batch_ldg_any_kernel(groups[i].cfg.k, groups[i].cfg.cta);
+            if (any && plan_ctas(any, groups[i], sms, &u.ctas) == SL_OK) {
+                for (size_t j = i; j < groups.size(); ++j)
+                    if (groups[j].entry == groups[i].entry && !groups[j].items.empty()) {
+                        u.groups.push_back(static_cast<int>(j));
+                        u.nitems += groups[j].items.size();
+                    }
+                if (u.groups.size() > 1 && u.nitems <= 2 * static_cast<uint64_t>(u.ctas)) u.fn = any;
+            }
+        }
+        if (!u.fn) {
+            u.fn = groups[i].fn;
+            u.groups.assign(1, static_cast<int>(i));
+            u.ctas = groups[i].ctas;
+            u.nitems = groups[i].items.size();
+        }
+        for (int j : u.groups) taken[j] = true;
+        units->push_back(u);
+    }
+    return SL_OK;
 }
 
 // Everything after the argument checks; the caller releases b on failure.
@@ -216,8 +264,8 @@ int build_batch(sl_batch* b, const sl_batch_desc* descs, int32_t n, const sl_tun
         b->groups[gidx[key]].bytes += d.bytes;
     }
 
-    // ---- items (buffers in order), then every group's place in the item and
-    // partial arrays, then each buffer's partial slots
+    // ---- items (buffers in order), then every launch's and group's place in the
+    // item and partial arrays, then each buffer's partial slots
     std::vector<uint64_t> first(n);  // index of the buffer's first item in its group
     for (int32_t i = 0; i < n; ++i) {
         Group& g = b->groups[b->class_of[i]];
@@ -228,18 +276,24 @@ int build_batch(sl_batch* b, const sl_batch_desc* descs, int32_t n, const sl_tun
             BatchItem it;
             it.ptr = reinterpret_cast<const uint4*>(p + off);
             it.nvec = static_cast<uint32_t>(std::min(step, bytes - off) / 16);
-            it.pad = 0;
+            it.dtype = static_cast<uint32_t>(descs[i].dtype);
             g.items.push_back(it);
         }
     }
     std::vector<BatchItem> all;
     uint64_t slots = 0;
-    for (Group& g : b->groups) {
-        g.item_off = all.size();
-        g.part_off = slots;
-        all.insert(all.end(), g.items.begin(), g.items.end());
-        slots += g.items.size() * g.slots;
-        g.grid = static_cast<int>(std::min<uint64_t>(g.ctas, g.items.size()));
+    std::vector<Unit> units;
+    const int prc = plan_units(b->groups, sms, &units);
+    if (prc) return prc;
+    for (Unit& u : units) {
+        u.item_off = all.size();
+        u.part_off = slots;
+        for (int j : u.groups) {
+            Group& g = b->groups[j];
+            g.part_off = slots;
+            all.insert(all.end(), g.items.begin(), g.items.end());
+            slots += g.items.size() * g.slots;
+        }
     }
     // (the kernels count items, claims past the last one included, and slots in 32 bits)
     if (slots >= (1ull << 31)) return bfail(SL_ERR_ARG, "batch too large");
@@ -252,8 +306,8 @@ int build_batch(sl_batch* b, const sl_batch_desc* descs, int32_t n, const sl_tun
     }
 
     // ---- device tables (allocated before capture)
-    const size_t ng = b->groups.size();
-    const size_t ctrl_bytes = (16 + ng) * sizeof(uint32_t);
+    const size_t nu = units.size();
+    const size_t ctrl_bytes = (16 + nu) * sizeof(uint32_t);
     B_TRY(cudaMalloc(&b->d_items, std::max<size_t>(all.size(), 1) * sizeof(BatchItem)), "cudaMalloc failed");
     B_TRY(cudaMalloc(&b->d_segs, std::max<size_t>(n, 1) * sizeof(BufSeg)), "cudaMalloc failed");
     B_TRY(cudaMalloc(&b->d_parts, std::max<uint64_t>(slots, 1) * sizeof(WarpPartial)), "cudaMalloc failed");
@@ -271,7 +325,7 @@ int build_batch(sl_batch* b, const sl_batch_desc* descs, int32_t n, const sl_tun
     B_TRY(cudaEventCreate(&b->e0), "event create failed");
     B_TRY(cudaEventCreate(&b->e1), "event create failed");
     B_TRY(cudaEventCreateWithFlags(&b->fork_ev, cudaEventDisableTiming), "event create failed");
-    for (size_t g = 0; g < ng; ++g) {
+    for (size_t g = 0; g < nu; ++g) {
         cudaStream_t s;
         cudaEvent_t e;
         B_TRY(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking), "stream create failed");
@@ -281,27 +335,29 @@ int build_batch(sl_batch* b, const sl_batch_desc* descs, int32_t n, const sl_tun
     }
     B_TRY(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal), "begin capture failed");
     cudaError_t ce = cudaEventRecord(b->fork_ev, b->stream);
-    for (size_t g = 0; g < ng && ce == cudaSuccess; ++g) {
-        Group& gr = b->groups[g];
+    for (size_t g = 0; g < nu && ce == cudaSuccess; ++g) {
+        const Unit& u = units[g];
+        const Group& gr = b->groups[u.groups[0]];
         ce = cudaStreamWaitEvent(b->branch[g], b->fork_ev, 0);
         if (ce != cudaSuccess) break;
         sl::BArgs a{};
-        a.items = b->d_items + gr.item_off;
-        a.nitems = static_cast<uint32_t>(gr.items.size());
+        a.items = b->d_items + u.item_off;
+        a.nitems = static_cast<uint32_t>(u.nitems);
         a.stage_bytes = static_cast<uint32_t>(gr.cfg.stage_bytes);
         a.next = b->d_ctrl + 16 + g;
-        a.parts = b->d_parts + gr.part_off;
+        a.parts = b->d_parts + u.part_off;
         a.err = b->d_ctrl;
         a.timeout_ns = TIMEOUT_NS;
         a.nst = gr.cfg.mech == SL_TMA ? gr.cfg.stages : 0;
         void* args[] = {&a};
-        if (a.nitems > 0) ce = cudaLaunchKernel(gr.fn, dim3(gr.grid), dim3(gr.block), args, gr.smem, b->branch[g]);
+        const unsigned grid = static_cast<unsigned>(std::min<uint64_t>(u.ctas, u.nitems));
+        ce = cudaLaunchKernel(u.fn, dim3(grid), dim3(gr.block), args, gr.smem, b->branch[g]);
         if (ce == cudaSuccess) ce = cudaEventRecord(b->branch_ev[g], b->branch[g]);
         if (ce == cudaSuccess) ce = cudaStreamWaitEvent(b->stream, b->branch_ev[g], 0);
     }
     if (ce == cudaSuccess)
         ce = sl::launch_batch_combine(b->d_segs, static_cast<uint32_t>(n), b->d_parts, b->d_ctrl, b->d_ctrl + 16,
-                                      static_cast<uint32_t>(ng), b->h_results, b->h_err, b->stream);
+                                      static_cast<uint32_t>(nu), b->h_results, b->h_err, b->stream);
     cudaGraph_t graph = nullptr;
     const cudaError_t ee = cudaStreamEndCapture(b->stream, &graph);
     b->graph = graph;

@@ -19,7 +19,7 @@ namespace sl {
 struct __align__(16) BatchItem {
     const uint4* ptr;  // first vector of the item
     uint32_t nvec;     // 16-byte vectors in the item (> 0)
-    uint32_t pad;
+    uint32_t dtype;    // sl_dtype of the buffer
 };
 static_assert(sizeof(BatchItem) == 16, "BatchItem layout");
 
@@ -59,14 +59,14 @@ __device__ __forceinline__ WarpPartial warp_partial(const Acc<DT>& acc) {
 }
 
 // The item loop of a class kernel whose CTAs work on one item together.
-// stream(item, acc) folds an item.  The next item's descriptor is copied to
+// stream(item) folds an item and returns the warp's partial.  The next item's descriptor is copied to
 // shared memory, and the one after it claimed, while the current item streams;
 // one CTA barrier per item publishes both together with the warps' partials,
 // which one warp (a different one for each item) then merges into the item's
 // partial while the others go on.  (Claiming, fetching the descriptor and two
 // barriers between items left every CTA idle for about 2 us per item.)  Little is kept in registers across stream():
 // the item's index and its place in the loop are re-read from shared memory.
-template <int DT, typename Stream>
+template <bool FLOATS, typename Stream>
 __device__ __forceinline__ void batch_items(const BArgs& a, Stream stream) {
     __shared__ BatchItem slot[2];
     __shared__ uint32_t sidx[3];
@@ -90,9 +90,7 @@ __device__ __forceinline__ void batch_items(const BArgs& a, Stream stream) {
             }
         }
         {
-            Acc<DT> acc;
-            stream(it, acc);
-            const WarpPartial w = warp_partial<DT>(acc);
+            const WarpPartial w = stream(it);
             if ((threadIdx.x & 31) == 0) wp[j & 1][threadIdx.x >> 5] = w;
         }
         if (threadIdx.x == 0) {
@@ -114,7 +112,7 @@ __device__ __forceinline__ void batch_items(const BArgs& a, Stream stream) {
                 hi = q.hi;
                 lo = q.lo;
             }
-            warp_merge<DT>(s, x, n, hi, lo);
+            warp_merge<FLOATS ? SL_F32 : SL_U32>(s, x, n, hi, lo);
             if (lane == 0) {
                 WarpPartial q;
                 q.sum = s;
@@ -131,39 +129,57 @@ __device__ __forceinline__ void batch_items(const BArgs& a, Stream stream) {
     }
 }
 
-// LDG class kernel: per item, tiles of CTA*K vectors, K independent 16-byte
-// loads per thread per tile (same fold and tile layout as k_ldg), guarded
-// ragged tail.
+// One item of an LDG class: tiles of CTA*K vectors, K independent 16-byte loads
+// per thread per tile (same fold and tile layout as k_ldg), guarded ragged tail.
+template <int K, int CTA, int DT>
+__device__ __forceinline__ WarpPartial ldg_item(const BatchItem& it) {
+    constexpr uint32_t TILE = static_cast<uint32_t>(CTA) * K;
+    Acc<DT> acc;
+    const uint32_t nfull = it.nvec / TILE;
+    const uint4* p = it.ptr + threadIdx.x;
+#pragma unroll 1
+    for (uint32_t t = 0; t < nfull; ++t, p += TILE) {
+        uint4 v[K];
+#pragma unroll
+        for (int k = 0; k < K; ++k) v[k] = ldg16<SL_COP_CG>(p + k * CTA);
+#pragma unroll
+        for (int k = 0; k < K; ++k) acc.fold(v[k]);
+    }
+    acc.n = nfull * K;
+    const uint32_t rem = it.nvec - nfull * TILE;
+    if (rem) {
+        uint4 v[K];
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            if (threadIdx.x + k * CTA < rem) v[k] = ldg16<SL_COP_CG>(p + k * CTA);
+            else v[k] = make_uint4(0u, 0u, 0u, 0u);
+        }
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            if (threadIdx.x + k * CTA < rem) {
+                acc.fold(v[k]);
+                acc.n += 1;
+            }
+        }
+    }
+    return warp_partial<DT>(acc);
+}
+
 template <int K, int CTA, int DT>
 __global__ void __launch_bounds__(CTA, DT == SL_BF16 ? ldg_min_blocks<K, CTA, DT>() : 1) kb_ldg(const BArgs a) {
-    constexpr uint32_t TILE = static_cast<uint32_t>(CTA) * K;
-    batch_items<DT>(a, [](const BatchItem& it, Acc<DT>& acc) {
-        const uint32_t nfull = it.nvec / TILE;
-        const uint4* p = it.ptr + threadIdx.x;
-#pragma unroll 1
-        for (uint32_t t = 0; t < nfull; ++t, p += TILE) {
-            uint4 v[K];
-#pragma unroll
-            for (int k = 0; k < K; ++k) v[k] = ldg16<SL_COP_CG>(p + k * CTA);
-#pragma unroll
-            for (int k = 0; k < K; ++k) acc.fold(v[k]);
-        }
-        acc.n = nfull * K;
-        const uint32_t rem = it.nvec - nfull * TILE;
-        if (rem) {
-            uint4 v[K];
-#pragma unroll
-            for (int k = 0; k < K; ++k) {
-                if (threadIdx.x + k * CTA < rem) v[k] = ldg16<SL_COP_CG>(p + k * CTA);
-                else v[k] = make_uint4(0u, 0u, 0u, 0u);
-            }
-#pragma unroll
-            for (int k = 0; k < K; ++k) {
-                if (threadIdx.x + k * CTA < rem) {
-                    acc.fold(v[k]);
-                    acc.n += 1;
-                }
-            }
+    batch_items<DT != SL_U32>(a, [](const BatchItem& it) { return ldg_item<K, CTA, DT>(it); });
+}
+
+// The LDG classes of one tuning entry, whatever their types, in one launch (the
+// host takes it for small classes: see plan_units in batch_api.cu).
+template <int K, int CTA>
+__global__ void __launch_bounds__(CTA) kb_ldg_any(const BArgs a) {
+    batch_items<true>(a, [](const BatchItem& it) {
+        switch (it.dtype) {
+        case SL_F32: return ldg_item<K, CTA, SL_F32>(it);
+        case SL_BF16: return ldg_item<K, CTA, SL_BF16>(it);
+        case SL_FP8_E4M3: return ldg_item<K, CTA, SL_FP8_E4M3>(it);
+        default: return ldg_item<K, CTA, SL_U32>(it);
         }
     });
 }

@@ -21,7 +21,8 @@ __global__ void __launch_bounds__(1024) kb_cpasync(const BArgs a) {
     extern __shared__ __align__(128) uint4 cp_ring[];  // [D][cta], 128-byte aligned (cp.async destinations)
     const uint32_t cta = blockDim.x, t = threadIdx.x;
     const uint32_t my0 = smem_addr(cp_ring + t), stride = cta * 16u;
-    batch_items<DT>(a, [&](const BatchItem& it, Acc<DT>& acc) {
+    batch_items<DT != SL_U32>(a, [&](const BatchItem& it) {
+        Acc<DT> acc;
         const uint32_t nchunks = (it.nvec + cta - 1) / cta;
         uint32_t islot = 0, cslot = 0;
 #pragma unroll
@@ -46,6 +47,7 @@ __global__ void __launch_bounds__(1024) kb_cpasync(const BArgs a) {
             cslot = (cslot + 1 == D) ? 0 : cslot + 1;
         }
         kb_cp_wait<0>();
+        return warp_partial<DT>(acc);
     });
 }
 

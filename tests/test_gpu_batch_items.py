@@ -83,3 +83,33 @@ def test_item_sums(sl, dtype, mech, kw, unit):
         assert abs(f - ref) <= 2e-6 * float(np.abs(v).sum())
         assert (su, xo) == oracle.checksum(part.view(np.uint32))
     sl.sl_batch_destroy(b)
+
+
+@pytest.mark.parametrize("k,cta", [(1, 512), (2, 128), (8, 256), (16, 128)])
+@pytest.mark.parametrize("scale", [1, 24])
+def test_mixed_types_of_one_entry(sl, k, cta, scale):
+    """Four types under one LDG entry: few items (one launch for all types) and
+    many (a launch per type); every result as that of its own buffer, in every
+    run."""
+    unit = k * cta * 16
+    kinds = [workloads.U32, workloads.F32, workloads.BF16, workloads.FP8_E4M3]
+    bufs, want = [], []
+    for i in range(16):
+        dt = kinds[i % 4]
+        nbytes = [16, unit - 16, unit + 16, 3 * unit * scale, 0][i % 5]
+        if dt == workloads.U32:
+            x = workloads.splitmix_u32(i + 1, nbytes // 4)
+        else:
+            x = workloads.payload(dt, nbytes // workloads.ELEM_BYTES[dt], seed=i + 1)
+        dev = torch.from_numpy(x.view(np.uint8).copy()).cuda()
+        ref = 0.0 if dt == workloads.U32 else oracle.fsum(dt, x)[0] if nbytes else 0.0
+        bufs.append((dev, nbytes, dt))
+        want.append((*(oracle.checksum(x.view(np.uint32)) if nbytes else (0, 0)), nbytes // 16, ref, nbytes))
+    b = sl.sl_batch_create(bufs, [sl.tune_entry(0, 1 << 62, sl.config("ldg", k=k, cta=cta))])
+    assert sl.sl_batch_info(b)[0] == 4
+    for _ in range(3):
+        for r, (s, x, n, f, nbytes) in zip(sl.sl_batch_run(b)[0], want):
+            assert (r.sum_u32, r.xor_u64, r.issued_loads, r.status) == (s, x, n, 0)
+            assert abs(r.fsum - f) <= 2e-6 * 448.0 * max(nbytes, 1)
+            assert abs(r.fsum - f) <= 2e-6 * max(abs(f), 1e-3 * 36.0 * max(nbytes, 1) ** 0.5)
+    sl.sl_batch_destroy(b)
