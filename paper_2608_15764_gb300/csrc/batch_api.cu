@@ -20,7 +20,7 @@ namespace sl {
 const void* batch_ldg_kernel(int dtype, int k, int cta);
 const void* batch_ldg_any_kernel(int k, int cta);
 const void* batch_cpasync_kernel(int dtype, int d);
-const void* batch_tma_kernel(int dtype, int batch);
+const void* batch_tma_kernel(int dtype, int batch, bool small_ring);
 cudaError_t launch_batch_combine(const BufSeg* segs, uint32_t nbuf, const WarpPartial* parts, uint32_t* err,
                                  uint32_t* next, uint32_t nclasses, sl_result* out, uint32_t* host_err,
                                  cudaStream_t s);
@@ -164,7 +164,8 @@ int plan_group(Group& g, int sms, int smem_optin) {
                          "(tma_ring must be SL_RING_CTA)");
         // consumer threads read their last 4 vectors of a stage (1 where they
         // read fewer) into registers before releasing it
-        g.fn = sl::batch_tma_kernel(g.dtype, c.stage_bytes / 16 >= 4 * c.cta ? 4 : 1);
+        g.fn = sl::batch_tma_kernel(g.dtype, c.stage_bytes / 16 >= 4 * c.cta ? 4 : 1,
+                                    static_cast<int64_t>(c.stages) * c.stage_bytes <= (56 << 10));
         g.block = c.cta + 32;
         g.smem = static_cast<size_t>(c.stages) * c.stage_bytes;
         g.slots = c.cta / 32;

@@ -41,8 +41,8 @@ struct BArgs {
 };
 
 // Reduce a warp's accumulators into one partial (lane 0 holds it afterwards).
-template <int DT>
-__device__ __forceinline__ WarpPartial warp_partial(const Acc<DT>& acc) {
+template <int DT, bool BIAS>
+__device__ __forceinline__ WarpPartial warp_partial(const Acc<DT, BIAS>& acc) {
     uint32_t s = acc.s;
     uint64_t x = (static_cast<uint64_t>(acc.xh) << 32) | acc.xl, n = acc.n;
     float hi = 0.0f, lo = 0.0f;
@@ -134,7 +134,7 @@ __device__ __forceinline__ void batch_items(const BArgs& a, Stream stream) {
 template <int K, int CTA, int DT>
 __device__ __forceinline__ WarpPartial ldg_item(const BatchItem& it) {
     constexpr uint32_t TILE = static_cast<uint32_t>(CTA) * K;
-    Acc<DT> acc;
+    Acc<DT, BIASED<DT, K>> acc;
     const uint32_t nfull = it.nvec / TILE;
     const uint4* p = it.ptr + threadIdx.x;
 #pragma unroll 1
@@ -142,8 +142,7 @@ __device__ __forceinline__ WarpPartial ldg_item(const BatchItem& it) {
         uint4 v[K];
 #pragma unroll
         for (int k = 0; k < K; ++k) v[k] = ldg16<SL_COP_CG>(p + k * CTA);
-#pragma unroll
-        for (int k = 0; k < K; ++k) acc.fold(v[k]);
+        acc.fold_n(v);
     }
     acc.n = nfull * K;
     const uint32_t rem = it.nvec - nfull * TILE;
@@ -162,7 +161,7 @@ __device__ __forceinline__ WarpPartial ldg_item(const BatchItem& it) {
             }
         }
     }
-    return warp_partial<DT>(acc);
+    return warp_partial(acc);
 }
 
 template <int K, int CTA, int DT>

@@ -47,7 +47,7 @@ __global__ void __launch_bounds__(1024) kb_cpasync(const BArgs a) {
             cslot = (cslot + 1 == D) ? 0 : cslot + 1;
         }
         kb_cp_wait<0>();
-        return warp_partial<DT>(acc);
+        return warp_partial(acc);
     });
 }
 
@@ -70,7 +70,7 @@ constexpr uint32_t STAGE_LAST_OF_ITEM = 1, STAGE_DONE = 2;
 // a consumer thread reads its last B vectors of a stage into registers and
 // its warp releases the stage before folding them (B = 4, or 1 where a
 // thread reads fewer than 4 vectors of a stage).
-template <int DT, int B>
+template <int DT, int B, bool BIAS>
 __global__ void __launch_bounds__(1024) kb_tma(const BArgs a) {
     extern __shared__ __align__(128) uint8_t tma_ring[];
     __shared__ __align__(8) uint64_t full[SL_MAX_STAGES];
@@ -148,7 +148,8 @@ __global__ void __launch_bounds__(1024) kb_tma(const BArgs a) {
         __syncwarp();
     } else {
         const uint32_t ct = threadIdx.x - 32, nct = ncw * 32;
-        Acc<DT> acc;
+        using TAcc = Acc<DT, BIAS>;
+        TAcc acc;
         uint32_t s = 0, r = 0;
         for (;;) {
             const bool got =
@@ -157,32 +158,60 @@ __global__ void __launch_bounds__(1024) kb_tma(const BArgs a) {
             const StageMeta m = meta[s];  // read before the stage is released
             if (m.flags & STAGE_DONE) break;
             const uint32_t base = ring0 + s * S;
-            uint32_t v = ct;
+            if constexpr (BIAS) {
+                // one place where vectors are folded together (its code is long)
+                for (uint32_t v0 = ct & ~31u;; v0 += B * nct) {  // warp-uniform
+                    const uint32_t v = v0 + lane;
+                    const bool last = v0 + B * nct >= m.nv;
+                    if (v0 + 31 + (B - 1) * nct < m.nv) {
+                        uint4 x[B];
+#pragma unroll
+                        for (int u = 0; u < B; ++u) x[u] = lds16(base + 16u * (v + u * nct));
+                        if (last) {
+                            __syncwarp();
+                            if (lane == 0) mbar_arrive(empty0 + 8 * s);
+                        }
+                        acc.fold_n(x);
+                        acc.n += B;
+                    } else {
 #pragma unroll 1
-            for (; v + B * nct < m.nv; v += B * nct) {
+                        for (uint32_t w = v; w < m.nv && w < v + B * nct; w += nct) {
+                            acc.fold(lds16(base + 16u * w));
+                            acc.n += 1;
+                        }
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(empty0 + 8 * s);
+                    }
+                    if (last) break;
+                }
+            } else {
+                uint32_t v = ct;
+#pragma unroll 1
+                for (; v + B * nct < m.nv; v += B * nct) {
+                    uint4 x[B];
+#pragma unroll
+                    for (int u = 0; u < B; ++u) x[u] = lds16(base + 16u * (v + u * nct));
+#pragma unroll
+                    for (int u = 0; u < B; ++u) acc.fold(x[u]);
+                    acc.n += B;
+                }
                 uint4 x[B];
 #pragma unroll
-                for (int u = 0; u < B; ++u) x[u] = lds16(base + 16u * (v + u * nct));
+                for (int u = 0; u < B; ++u)
+                    if (v + u * nct < m.nv) x[u] = lds16(base + 16u * (v + u * nct));
+                __syncwarp();
+                if (lane == 0) mbar_arrive(empty0 + 8 * s);
 #pragma unroll
-                for (int u = 0; u < B; ++u) acc.fold(x[u]);
-                acc.n += B;
+                for (int u = 0; u < B; ++u)
+                    if (v + u * nct < m.nv) {
+                        acc.fold(x[u]);
+                        acc.n += 1;
+                    }
             }
-            uint4 x[B];
-#pragma unroll
-            for (int u = 0; u < B; ++u)
-                if (v + u * nct < m.nv) x[u] = lds16(base + 16u * (v + u * nct));
-            __syncwarp();
-            if (lane == 0) mbar_arrive(empty0 + 8 * s);
-#pragma unroll
-            for (int u = 0; u < B; ++u)
-                if (v + u * nct < m.nv) {
-                    acc.fold(x[u]);
-                    acc.n += 1;
-                }
             if (m.flags & STAGE_LAST_OF_ITEM) {
-                const WarpPartial w = warp_partial<DT>(acc);
+                const WarpPartial w = warp_partial(acc);
                 if (lane == 0) a.parts[static_cast<size_t>(m.item) * ncw + (warp - 1)] = w;
-                acc = Acc<DT>();
+                acc = TAcc();
             }
             if (++s == nst) { s = 0; ++r; }
         }
@@ -285,16 +314,18 @@ const void* batch_cpasync_kernel(int dtype, int d) {
 template <int B>
 static const void* kb_tma_b(int dtype) {
     switch (dtype) {
-    case SL_U32: return reinterpret_cast<const void*>(&kb_tma<SL_U32, B>);
-    case SL_F32: return reinterpret_cast<const void*>(&kb_tma<SL_F32, B>);
-    case SL_BF16: return reinterpret_cast<const void*>(&kb_tma<SL_BF16, B>);
-    case SL_FP8_E4M3: return reinterpret_cast<const void*>(&kb_tma<SL_FP8_E4M3, B>);
+    case SL_U32: return reinterpret_cast<const void*>(&kb_tma<SL_U32, B, false>);
+    case SL_F32: return reinterpret_cast<const void*>(&kb_tma<SL_F32, B, false>);
+    case SL_BF16: return reinterpret_cast<const void*>(&kb_tma<SL_BF16, B, false>);
+    case SL_FP8_E4M3: return reinterpret_cast<const void*>(&kb_tma<SL_FP8_E4M3, B, false>);
     default: return nullptr;
     }
 }
 
-const void* batch_tma_kernel(int dtype, int batch) {
-    if (batch == 4) return kb_tma_b<4>(dtype);
+const void* batch_tma_kernel(int dtype, int batch, bool small_ring) {
+    if (batch == 4)
+        return dtype == SL_BF16 && small_ring ? reinterpret_cast<const void*>(&kb_tma<SL_BF16, 4, true>)
+                                              : kb_tma_b<4>(dtype);
     if (batch == 1) return kb_tma_b<1>(dtype);
     return nullptr;
 }

@@ -42,7 +42,9 @@ __global__ void __launch_bounds__(D * G > 8 ? 512 : 1024) k_cpasync_dyn(const KA
         len = left < chunk_vec ? static_cast<uint32_t>(left) : chunk_vec;
         p = buf + base + threadIdx.x;
     };
-    Acc<DT> acc;
+    // (groups of copies folded together where the registers allow it)
+    constexpr bool BIAS = BIASED<DT, G> && (D * G > 8);
+    Acc<DT, BIAS> acc;
     uint32_t full_tiles = 0;
     volatile uint32_t* vs = slot;
     if (threadIdx.x == 0) vs[1] = dyn_claim(a);  // on its way during the prologue
@@ -91,8 +93,15 @@ __global__ void __launch_bounds__(D * G > 8 ? 512 : 1024) k_cpasync_dyn(const KA
 #pragma unroll
                 for (int k = 0; k < D; ++k) {
                     cp_async_wait<D - 1>();
+                    if constexpr (BIAS) {
+                        uint4 w[G];
 #pragma unroll
-                    for (int g = 0; g < G; ++g) acc.fold(lds16(my0 + (k * G + g) * stride));
+                        for (int g = 0; g < G; ++g) w[g] = lds16(my0 + (k * G + g) * stride);
+                        acc.fold_n(w);
+                    } else {
+#pragma unroll
+                        for (int g = 0; g < G; ++g) acc.fold(lds16(my0 + (k * G + g) * stride));
+                    }
 #pragma unroll
                     for (int g = 0; g < G; ++g) {
                         const uint32_t j = k * G + g;
@@ -135,7 +144,7 @@ __global__ void __launch_bounds__(D * G > 8 ? 512 : 1024) k_cpasync_dyn(const KA
     }
     cp_async_wait<0>();
     acc.n += full_tiles * (D * G);
-    cta_finish<DT>(acc, true, threadIdx.x >> 5, cta >> 5, a);
+    cta_finish(acc, true, threadIdx.x >> 5, cta >> 5, a);
 }
 
 template <int D, int G, int DT>

@@ -30,7 +30,7 @@ __global__ void __launch_bounds__(CTA, ldg_min_blocks<K, CTA, DT>()) k_ldg(const
     const uint32_t ntiles = static_cast<uint32_t>(a.ntiles);
     const uint32_t total = static_cast<uint32_t>(a.total);
     const bool last_full = (a.nvec == static_cast<uint64_t>(ntiles) * TILE);
-    Acc<DT> acc;
+    Acc<DT, BIASED<DT, K>> acc;
     uint32_t full_iters = 0;
     TileCursor c;
     c.start(ntiles);
@@ -47,8 +47,7 @@ __global__ void __launch_bounds__(CTA, ldg_min_blocks<K, CTA, DT>()) k_ldg(const
 #pragma unroll
                 for (int k = 0; k < K; ++k) cov_count<COV>(a, (p + k * CTA) - buf);
             }
-#pragma unroll
-            for (int k = 0; k < K; ++k) acc.fold(v[k]);
+            acc.fold_n(v);
             ++full_iters;
         } else {
             // Ragged last tile: only vectors below nvec are loaded.
@@ -72,7 +71,7 @@ __global__ void __launch_bounds__(CTA, ldg_min_blocks<K, CTA, DT>()) k_ldg(const
         }
     }
     acc.n += full_iters * K;
-    cta_finish<DT>(acc, true, threadIdx.x >> 5, CTA / 32, a);
+    cta_finish(acc, true, threadIdx.x >> 5, CTA / 32, a);
 }
 
 // SL_DYN traversal: CTAs claim contiguous chunks of a.tile_vec vectors (a
@@ -93,7 +92,7 @@ __global__ void __launch_bounds__(CTA, ldg_min_blocks<K, CTA, DT>()) k_ldg_dyn(c
     const uint4* __restrict__ buf = static_cast<const uint4*>(a.buf);
     const uint32_t chunk_vec = a.tile_vec;
     const uint32_t total = static_cast<uint32_t>(a.total);
-    Acc<DT> acc;
+    Acc<DT, BIASED<DT, K>> acc;
     uint32_t full_iters = 0;
     volatile uint32_t* vslot = slot;
     uint32_t cur = dyn_first();
@@ -114,8 +113,7 @@ __global__ void __launch_bounds__(CTA, ldg_min_blocks<K, CTA, DT>()) k_ldg_dyn(c
 #pragma unroll
                 for (int k = 0; k < K; ++k) cov_count<COV>(a, (p + k * CTA) - buf);
             }
-#pragma unroll
-            for (int k = 0; k < K; ++k) acc.fold(v[k]);
+            acc.fold_n(v);
         }
         full_iters += nfull;
         const uint32_t rem = len - nfull * TILE;
@@ -142,7 +140,7 @@ __global__ void __launch_bounds__(CTA, ldg_min_blocks<K, CTA, DT>()) k_ldg_dyn(c
         cur = vslot[(j + 1) & 1];
     }
     acc.n += full_iters * K;
-    cta_finish<DT>(acc, true, threadIdx.x >> 5, CTA / 32, a);
+    cta_finish(acc, true, threadIdx.x >> 5, CTA / 32, a);
 }
 
 }  // namespace sl

@@ -31,11 +31,22 @@ __device__ __forceinline__ Oct ldg32(const Oct* p) {
     return v;
 }
 
+template <typename A, int K>
+__device__ __forceinline__ void fold_octs(A& acc, const Oct (&v)[K]) {
+    uint4 w[2 * K];
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        w[2 * k] = v[k].lo;
+        w[2 * k + 1] = v[k].hi;
+    }
+    acc.fold_n(w);
+}
+
 // Guarded tail of a tile or chunk: units below n32 load 32 bytes, the unit
 // n32 itself (when the buffer ends in a half unit) loads the last 16 bytes.
 template <int K, int CTA, int DT, bool COV>
 __device__ __forceinline__ void ragged32(const KArgs& a, const Oct* buf, uint64_t first, uint64_t n32, bool half,
-                                         Acc<DT>& acc) {
+                                         Acc<DT, BIASED<DT, 2 * K>>& acc) {
 #pragma unroll 1
     for (int k = 0; k < K; ++k) {
         const uint64_t u = first + static_cast<uint64_t>(k) * CTA + threadIdx.x;
@@ -64,7 +75,7 @@ __global__ void __launch_bounds__(CTA, 1) k_ldg32(const KArgs a) {
     const uint32_t ntiles = static_cast<uint32_t>(a.ntiles);
     const uint32_t total = static_cast<uint32_t>(a.total);
     const bool last_full = !half && n32 == static_cast<uint64_t>(ntiles) * TILE;
-    Acc<DT> acc;
+    Acc<DT, BIASED<DT, 2 * K>> acc;
     uint32_t full_iters = 0;
     TileCursor c;
     c.start(ntiles);
@@ -83,18 +94,14 @@ __global__ void __launch_bounds__(CTA, 1) k_ldg32(const KArgs a) {
                     cov_count<COV>(a, 2 * static_cast<uint64_t>((p + k * CTA) - buf) + 1);
                 }
             }
-#pragma unroll
-            for (int k = 0; k < K; ++k) {
-                acc.fold(v[k].lo);
-                acc.fold(v[k].hi);
-            }
+            fold_octs(acc, v);
             ++full_iters;
         } else {
             ragged32<K, CTA, DT, COV>(a, buf, static_cast<uint64_t>(tile) * TILE, n32, half, acc);
         }
     }
     acc.n += full_iters * K;
-    cta_finish<DT>(acc, true, threadIdx.x >> 5, CTA / 32, a);
+    cta_finish(acc, true, threadIdx.x >> 5, CTA / 32, a);
 }
 
 // SL_DYN: chunks of a.tile_vec units claimed from *a.next (the next claim
@@ -112,7 +119,7 @@ __global__ void __launch_bounds__(CTA, K == 1 ? (DT == SL_U32 ? 2048 : 1280) / C
     const uint64_t units = n32 + (half ? 1 : 0);
     const uint32_t chunk = a.tile_vec;
     const uint32_t total = static_cast<uint32_t>(a.total);
-    Acc<DT> acc;
+    Acc<DT, BIASED<DT, 2 * K>> acc;
     volatile uint32_t* vslot = slot;
     uint32_t cur = dyn_first();
 #pragma unroll 1
@@ -137,11 +144,7 @@ __global__ void __launch_bounds__(CTA, K == 1 ? (DT == SL_U32 ? 2048 : 1280) / C
                     cov_count<COV>(a, 2 * static_cast<uint64_t>((p + k * CTA) - buf) + 1);
                 }
             }
-#pragma unroll
-            for (int k = 0; k < K; ++k) {
-                acc.fold(v[k].lo);
-                acc.fold(v[k].hi);
-            }
+            fold_octs(acc, v);
         }
         acc.n += nfull * K;
         if (nfull * TILE < len)
@@ -149,7 +152,7 @@ __global__ void __launch_bounds__(CTA, K == 1 ? (DT == SL_U32 ? 2048 : 1280) / C
         __syncthreads();  // the prefetched claim is visible; the slot read next is not rewritten until j+2
         cur = vslot[(j + 1) & 1];
     }
-    cta_finish<DT>(acc, true, threadIdx.x >> 5, CTA / 32, a);
+    cta_finish(acc, true, threadIdx.x >> 5, CTA / 32, a);
 }
 
 template <int CTA, int DT, bool DYN>

@@ -68,7 +68,7 @@ __global__ void __launch_bounds__(CTA, 1) k_ldg4(const KArgs a) {
     acc.xl = (threadIdx.x & 1) ? 0u : xr;
     acc.xh = (threadIdx.x & 1) ? xr : 0u;
     acc.n = n + full_iters * K;
-    cta_finish<SL_U32>(acc, true, threadIdx.x >> 5, CTA / 32, a);
+    cta_finish(acc, true, threadIdx.x >> 5, CTA / 32, a);
 }
 
 template <int CTA>

@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(CTA, 1) k_ldg_fixed(const KArgs a) {
         }
     }
     acc.n = iters * K;
-    cta_finish<SL_U32>(acc, true, threadIdx.x >> 5, CTA / 32, a);
+    cta_finish(acc, true, threadIdx.x >> 5, CTA / 32, a);
 }
 
 template <int CTA>

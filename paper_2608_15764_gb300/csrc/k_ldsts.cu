@@ -67,7 +67,7 @@ __global__ void __launch_bounds__(G <= 8 ? 1024 : 256, 1) k_ldsts(const KArgs a)
         }
     }
     acc.n += full_iters * G;
-    cta_finish<DT>(acc, true, threadIdx.x >> 5, cta >> 5, a);
+    cta_finish(acc, true, threadIdx.x >> 5, cta >> 5, a);
 }
 
 template <int DT>

@@ -141,7 +141,7 @@ __global__ void __launch_bounds__(1024, 1) k_tma(const KArgs a) {
         }
     }
     // consumer warps fold (all lanes left the ring together); warp 0 does not
-    cta_finish<DT>(acc, warp != 0, warp - 1, ncw, a, &cta_err);
+    cta_finish(acc, warp != 0, warp - 1, ncw, a, &cta_err);
 }
 
 // ---- k_tma_warp: the CTA's stages dealt to its warps (SL_RING_WARP) ----
@@ -297,7 +297,7 @@ __global__ void __launch_bounds__(SL_MAX_STAGES * 32, 4) k_tma_warp(const KArgs 
                              DEV_ERR_TIMEOUT_DRAIN);
     }
     __syncwarp();
-    cta_finish<DT>(acc, true, warp, nw, a, &cta_err);
+    cta_finish(acc, true, warp, nw, a, &cta_err);
 }
 
 const void* tma_cov_kernel(int batch) {

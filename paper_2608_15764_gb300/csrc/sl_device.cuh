@@ -119,6 +119,17 @@ __device__ __forceinline__ void cov_count(const KArgs& a, uint64_t i) {
     if constexpr (COV) atomicAdd(a.cov + i, 1u);
 }
 
+// Largest of each 16-bit half.
+__device__ __forceinline__ uint32_t max_u16x2(uint32_t a, uint32_t b) {
+    uint32_t d;
+    asm("max.u16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
+    return d;
+}
+
+// Whether a kernel that folds n vectors at a time takes the biased sum.
+template <int DT, int N>
+constexpr bool BIASED = DT == SL_BF16 && N >= 4 && N <= 16;
+
 // ---- the fold ----------------------------------------------------------------
 // Per-thread accumulator.  Integer part (every dtype): wraparound uint32 sum
 // of the four words and XOR of the two little-endian uint64 halves.
@@ -136,11 +147,34 @@ __device__ __forceinline__ void cov_count(const KArgs& a, uint64_t i) {
 //         vector is left uncompensated, whatever the values' range;
 //   FP8:  the two half-vector sums, each exact (fp8_word_sum), go through one
 //         packed TwoSum step.
-template <int DT>
+//
+// BIAS (BF16 where a thread folds four or more vectors at a time, fold_n): the
+// running sum is held as fs = C + sum with a power-of-two bias C = 1.5 * 2^k
+// well above the data, so that |fs| >= |x| in every addition and its rounding
+// error needs the three operations of Dekker's Fast2Sum where TwoSum needs six:
+// 16 packed operations per vector instead of 28.  fold_n looks at the largest
+// exponent of its vectors first: C is 2^9 to 2^11 times the largest value of the
+// first ones (a running sum of a few thousand values grows to that too, so the
+// errors collected in fe are of the size that TwoSum's are), is raised when the
+// sum itself has grown to a quarter of it, and a thread that meets values of
+// different sizes (the largest of two vectors 2^5 apart from that of all) when
+// it takes a C, a value too large for the C it has, an infinity or a NaN goes on
+// with TwoSum (c = SLOW); a single vector is added by TwoSum.  fs - C is exact, so
+// entering and leaving lose nothing.
+// Measured, TwoSum then biased: 16 passes over 32 MiB in L2 at K = 8 73.5 ->
+// 65.7 us, 48 MiB by cp.async 2 x 8 14.7 -> 13.7, 4 GiB at K = 8 dynamic 584 ->
+// 576, 1,024 buffers of 16 GiB 2,555 -> 2,425 on the device.  Sums of N(0,1)
+// values are exact to the last bit of the FP64 result either way; where the
+// data's size drops by 2^17 half way, 1e-13 of sum|x| (TwoSum 1e-15).  Kernels
+// with fewer vectors at a time (K < 4, one copy per group) or few warps per SM
+// (the 64 KiB TMA rings: 177 -> 200 us per GiB) stay with TwoSum.
+template <int DT, bool BIAS = false>
 struct Acc {
+    static constexpr uint32_t SLOW = 0xFFFFFFFFu;
     uint32_t s = 0, xl = 0, xh = 0;
     uint32_t n = 0;  // 16-byte loads folded by this thread (the host keeps it below 2^32)
     uint64_t fs = 0, fe = 0;  // packed (lane 0, lane 1) running sums and error sums; 0 bits = +0.0f
+    uint32_t c = 0;           // BIAS: bits of C in both lanes of fs; 0: none now; SLOW: none from here on
 
     // TwoSum of the packed pair x into (fs, fe), lane by lane.
     __device__ __forceinline__ void add2(uint64_t x) {
@@ -152,10 +186,124 @@ struct Acc {
         fs = t;
     }
 
-    __device__ __forceinline__ void fold(const uint4& v) {
+    // As add2 where |fs| >= |x| in both lanes (Fast2Sum).
+    __device__ __forceinline__ void add2_biased(uint64_t x) {
+        const uint64_t t = f2_add(fs, x);
+        fe = f2_add(fe, f2_sub(x, f2_sub(t, fs)));
+        fs = t;
+    }
+
+    __device__ __forceinline__ void leave_bias() {
+        if (c != 0 && c != SLOW) {
+            fs = f2_sub(fs, f2_pack(c, c));
+            c = 0;
+        }
+    }
+
+    // Take a bias for values of biased exponents up to e.  head: what C's
+    // exponent is above that of the largest value that one fold_n may add.
+    __device__ __forceinline__ void enter_bias(uint32_t e, uint32_t head) {
+        const uint32_t f0 = (static_cast<uint32_t>(fs) >> 23) & 255u;
+        const uint32_t f1 = (static_cast<uint32_t>(fs >> 32) >> 23) & 255u;
+        uint32_t k = e + head + 2;  // values may grow fourfold
+        const uint32_t f = (f0 > f1 ? f0 : f1) + 3;
+        k = k > f ? k : f;
+        if (k > 240u) {
+            c = SLOW;
+            return;
+        }
+        c = (k << 23) | 0x400000u;
+        const uint64_t old = fs;
+        fs = f2_pack(c, c);
+        add2_biased(old);
+    }
+
+    // Largest code of two vectors' values, signs left out (volatile: computed
+    // where it is needed, not shared with fold_n's own maximum at the price of
+    // registers).
+    static __device__ __forceinline__ uint32_t pair_code(const uint4& a, const uint4& b) {
+        uint32_t m = 0;
+        const uint32_t w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            asm volatile("{\n\t.reg .b32 t;\n\tand.b32 t, %1, 0x7FFF7FFF;\n\tmax.u16x2 %0, %0, t;\n\t}"
+                         : "+r"(m) : "r"(w[i]));
+        return m >> 16 > (m & 0xFFFFu) ? m >> 16 : m & 0xFFFFu;
+    }
+
+    // N vectors at once (N <= 16), by all lanes of the warp together.
+    template <int N>
+    __device__ __forceinline__ void fold_n(const uint4 (&v)[N]) {
+        if constexpr (!BIAS) {
+#pragma unroll
+            for (int i = 0; i < N; ++i) fold(v[i]);
+        } else {
+            // 4N additions per lane, below 2^(log2(4N) + 1) of the largest value's
+            // power of two, move fs by at most a quarter of 2^k
+            constexpr uint32_t HEAD = N > 8 ? 9 : N > 4 ? 8 : 7;
+#pragma unroll
+            for (int i = 0; i < N; ++i) fold_int(v[i]);
+            if (c != SLOW) {
+                uint32_t m = 0;
+#pragma unroll
+                for (int i = 0; i < N; ++i) {
+                    m = max_u16x2(m, v[i].x & 0x7FFF7FFFu);
+                    m = max_u16x2(m, v[i].y & 0x7FFF7FFFu);
+                    m = max_u16x2(m, v[i].z & 0x7FFF7FFFu);
+                    m = max_u16x2(m, v[i].w & 0x7FFF7FFFu);
+                }
+                m = m >> 16 > (m & 0xFFFFu) ? m >> 16 : m & 0xFFFFu;
+                const uint32_t e = m >> 7;
+                // bits 22 and 21 differ while fs is between 1.25 and 1.75 * 2^k
+                const uint32_t w0 = static_cast<uint32_t>(fs), w1 = static_cast<uint32_t>(fs >> 32);
+                const bool far = ((w0 ^ (w0 << 1)) & (w1 ^ (w1 << 1)) & 0x400000u) == 0;
+                if (c == 0 || far || e + HEAD > c >> 23) {
+                    // no bias yet, the sum has outgrown it, or the values have
+                    const bool larger = c != 0 && !far && !(fs == f2_pack(c, c) && fe == 0);
+                    leave_bias();
+                    // values of one size only: beside a lone large one the others
+                    // would be summed in fe alone
+                    const uint32_t p = pair_code(v[0], v[1]), q = pair_code(v[2], v[3]);
+                    const uint32_t least = (p < q ? p : q) >> 7;
+                    if (larger || (least != 0 && e > least + 4)) c = SLOW;
+                    else enter_bias(e, HEAD);
+                    if (c != SLOW && e + HEAD > c >> 23) {
+                        leave_bias();
+                        c = SLOW;
+                    }
+                }
+            }
+            // One lane on the long way takes its warp along: both ways would be run.
+            if (!__any_sync(FULL_MASK, c == SLOW)) {
+#pragma unroll
+                for (int i = 0; i < N; ++i) {
+                    add2_biased(f2_pack(v[i].x << 16, v[i].x & 0xFFFF0000u));
+                    add2_biased(f2_pack(v[i].y << 16, v[i].y & 0xFFFF0000u));
+                    add2_biased(f2_pack(v[i].z << 16, v[i].z & 0xFFFF0000u));
+                    add2_biased(f2_pack(v[i].w << 16, v[i].w & 0xFFFF0000u));
+                }
+            } else {
+                leave_bias();
+                c = SLOW;
+#pragma unroll
+                for (int i = 0; i < N; ++i) fold_float(v[i]);
+            }
+        }
+    }
+
+    __device__ __forceinline__ void fold_int(const uint4& v) {
         s += (v.x + v.y) + (v.z + v.w);
         xl ^= v.x ^ v.z;
         xh ^= v.y ^ v.w;
+    }
+
+    __device__ __forceinline__ void fold(const uint4& v) {
+        if constexpr (BIAS) leave_bias();
+        fold_int(v);
+        fold_float(v);
+    }
+
+    __device__ __forceinline__ void fold_float(const uint4& v) {
         if constexpr (DT == SL_F32) {
             add2(f2_pack(v.x, v.y));
             add2(f2_pack(v.z, v.w));
@@ -194,11 +342,14 @@ __device__ __forceinline__ void df_add(float& hi, float& lo, float ohi, float ol
     lo = se - (hi - sh);
 }
 
-template <int DT>
-__device__ __forceinline__ void Acc<DT>::float_part(float& hi, float& lo) const {
-    hi = f2_lane0(fs);
+template <int DT, bool BIAS>
+__device__ __forceinline__ void Acc<DT, BIAS>::float_part(float& hi, float& lo) const {
+    uint64_t f = fs;
+    if constexpr (BIAS)
+        if (c != 0 && c != SLOW) f = f2_sub(f, f2_pack(c, c));
+    hi = f2_lane0(f);
     lo = f2_lane0(fe);
-    df_add(hi, lo, f2_lane1(fs), f2_lane1(fe));
+    df_add(hi, lo, f2_lane1(f), f2_lane1(fe));
 }
 
 // ---- warp reductions ------------------------------------------------------------
@@ -336,8 +487,8 @@ __device__ __forceinline__ uint64_t& cta_start_stamp() {
 // final_combine.  `fw` is
 // this warp's index among the nfw (<= 32) folding warps; `cta_err`, if given,
 // is a CTA-local error code (shared memory) that thread 0 publishes to *a.err.
-template <int DT>
-__device__ __forceinline__ void cta_finish(const Acc<DT>& acc, bool folds, uint32_t fw, uint32_t nfw,
+template <int DT, bool BIAS = false>
+__device__ __forceinline__ void cta_finish(const Acc<DT, BIAS>& acc, bool folds, uint32_t fw, uint32_t nfw,
                                            const KArgs& a, const uint32_t* cta_err = nullptr) {
     __shared__ WarpPartial sp[32];
     const uint32_t lane = threadIdx.x & 31;
