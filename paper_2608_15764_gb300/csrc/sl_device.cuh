@@ -152,7 +152,7 @@ constexpr bool BIASED = DT == SL_BF16 && N >= 4 && N <= 16;
 // running sum is held as fs = C + sum with a power-of-two bias C = 1.5 * 2^k
 // well above the data, so that |fs| >= |x| in every addition and its rounding
 // error needs the three operations of Dekker's Fast2Sum where TwoSum needs six:
-// 16 packed operations per vector instead of 28.  fold_n looks at the largest
+// 16 packed operations per vector (and three per fold_n) instead of 28.  fold_n looks at the largest
 // exponent of its vectors first: C is 2^9 to 2^11 times the largest value of the
 // first ones (a running sum of a few thousand values grows to that too, so the
 // errors collected in fe are of the size that TwoSum's are), is raised when the
@@ -163,11 +163,11 @@ constexpr bool BIASED = DT == SL_BF16 && N >= 4 && N <= 16;
 // entering and leaving lose nothing.
 // Measured, TwoSum then biased: 16 passes over 32 MiB in L2 at K = 8 73.5 ->
 // 65.7 us, 48 MiB by cp.async 2 x 8 14.7 -> 13.7, 4 GiB at K = 8 dynamic 584 ->
-// 576, 1,024 buffers of 16 GiB 2,555 -> 2,425 on the device.  Sums of N(0,1)
-// values are exact to the last bit of the FP64 result either way; where the
-// data's size drops by 2^17 half way, 1e-13 of sum|x| (TwoSum 1e-15).  Kernels
-// with fewer vectors at a time (K < 4, one copy per group) or few warps per SM
-// (the 64 KiB TMA rings: 177 -> 200 us per GiB) stay with TwoSum.
+// 576, 1,024 buffers of 16 GiB 2,555 -> 2,440 on the device.  Errors against 64
+// bits: 0 either way on N(0,1) values (256 MiB and 16 GiB); where the data's size
+// drops by 2^17 half way, 3e-15 of sum|x| (TwoSum 1e-15).  Kernels with fewer
+// vectors at a time (K < 4, one copy per group) or few warps per SM (the 64 KiB
+// TMA rings: 177 -> 200 us per GiB) stay with TwoSum.
 template <int DT, bool BIAS = false>
 struct Acc {
     static constexpr uint32_t SLOW = 0xFFFFFFFFu;
@@ -282,6 +282,12 @@ struct Acc {
                     add2_biased(f2_pack(v[i].z << 16, v[i].z & 0xFFFF0000u));
                     add2_biased(f2_pack(v[i].w << 16, v[i].w & 0xFFFF0000u));
                 }
+                // what has become large enough of fe goes back to fs (exactly), so
+                // that fe stays below a few units in the last place of fs and its
+                // own roundings are no larger than under TwoSum
+                const uint64_t t = f2_add(fs, fe);
+                fe = f2_sub(fe, f2_sub(t, fs));
+                fs = t;
             } else {
                 leave_bias();
                 c = SLOW;
