@@ -152,15 +152,15 @@ constexpr bool BIASED = DT == SL_BF16 && N >= 4 && N <= 16;
 // running sum is held as fs = C + sum with a power-of-two bias C = 1.5 * 2^k
 // well above the data, so that |fs| >= |x| in every addition and its rounding
 // error needs the three operations of Dekker's Fast2Sum where TwoSum needs six:
-// 16 packed operations per vector (and three per fold_n) instead of 28.  fold_n looks at the largest
-// exponent of its vectors first: C is 2^9 to 2^11 times the largest value of the
-// first ones (a running sum of a few thousand values grows to that too, so the
-// errors collected in fe are of the size that TwoSum's are), is raised when the
-// sum itself has grown to a quarter of it, and a thread that meets values of
-// different sizes (the largest of two vectors 2^5 apart from that of all) when
-// it takes a C, a value too large for the C it has, an infinity or a NaN goes on
-// with TwoSum (c = SLOW); a single vector is added by TwoSum.  fs - C is exact, so
-// entering and leaving lose nothing.
+// 16 packed operations per vector (and three per fold_n) instead of 28.
+// fold_n looks at the largest exponent of its vectors first: C is 2^9 to 2^11
+// times the largest value of the first ones (a running sum of a few thousand
+// values grows to that too, so the errors collected in fe are of the size that
+// TwoSum's are), is raised when the sum itself has grown to a quarter of it, and
+// a thread that meets values of different sizes (the largest of two vectors 2^5
+// apart from that of all) when it takes a C, a value too large for the C it has,
+// an infinity or a NaN goes on with TwoSum (c = SLOW); a single vector is added by
+// TwoSum.  fs - C is exact, so entering and leaving lose nothing.
 // Measured, TwoSum then biased: 16 passes over 32 MiB in L2 at K = 8 73.5 ->
 // 65.7 us, 48 MiB by cp.async 2 x 8 14.7 -> 13.7, 4 GiB at K = 8 dynamic 584 ->
 // 576, 1,024 buffers of 16 GiB 2,555 -> 2,440 on the device.  Errors against 64
