@@ -66,10 +66,17 @@ __device__ __forceinline__ WarpPartial warp_partial(const Acc<DT, BIAS>& acc) {
 // partial while the others go on.  (Claiming, fetching the descriptor and two
 // barriers between items left every CTA idle for about 2 us per item.)  Little is kept in registers across stream():
 // the item's index and its place in the loop are re-read from shared memory.
+//
+// What orders the shared words, with B(j) the barrier of iteration j: a word is
+// written before B(j) and read after it, and its readers are done only at
+// B(j + 1).  Between B(j) and B(j + 1) warps read indices j and j + 1 while
+// thread 0 writes index j + 3, so there are four index words (with three,
+// index j + 3 would be index j's); they read descriptor j + 1 and partials j
+// while descriptor j + 2 and partials j + 1 are written: two of each.
 template <bool FLOATS, typename Stream>
 __device__ __forceinline__ void batch_items(const BArgs& a, Stream stream) {
     __shared__ BatchItem slot[2];
-    __shared__ uint32_t sidx[3];
+    __shared__ uint32_t sidx[4];
     __shared__ WarpPartial wp[2][32];
     volatile uint32_t* vidx = sidx;
     if (threadIdx.x == 0) {
@@ -79,10 +86,10 @@ __device__ __forceinline__ void batch_items(const BArgs& a, Stream stream) {
     BatchItem it = a.items[dyn_first()];
 #pragma unroll 1
     for (uint32_t j = 0;; ++j) {
-        // sidx[j % 3]: this item, [(j + 1) % 3]: the next, [(j + 2) % 3]: being claimed
+        // sidx[j & 3]: this item, [(j + 1) & 3]: the next, [(j + 2) & 3]: being claimed
         uint32_t claim = 0xFFFFFFFFu;
         if (threadIdx.x == 0) {
-            const uint32_t ahead = vidx[(j + 1) % 3];
+            const uint32_t ahead = vidx[(j + 1) & 3];
             if (ahead < a.nitems) {
                 asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(&slot[(j + 1) & 1])),
                              "l"(a.items + ahead) : "memory");
@@ -95,10 +102,10 @@ __device__ __forceinline__ void batch_items(const BArgs& a, Stream stream) {
         }
         if (threadIdx.x == 0) {
             asm volatile("cp.async.wait_all;" ::: "memory");
-            vidx[(j + 2) % 3] = claim;
+            vidx[(j + 2) & 3] = claim;
         }
         __syncthreads();
-        const uint32_t cur = vidx[j % 3], next = vidx[(j + 1) % 3];
+        const uint32_t cur = vidx[j & 3], next = vidx[(j + 1) & 3];
         const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
         if (warp == j % nw) {
             uint32_t s = 0;
