@@ -42,8 +42,9 @@ __global__ void __launch_bounds__(D * G > 8 ? 512 : 1024) k_cpasync(const KArgs 
     const uint64_t tile_vec = static_cast<uint64_t>(cta) * (D * G);
     const uint32_t skew = (static_cast<uint32_t>(a.debug) >> SL_DEBUG_SMEM_SKEW_SHIFT) & 7u;
     const uint32_t my0 = smem_addr(ring + skew + threadIdx.x), stride = cta * 16u;
-    // (groups of copies folded together where the registers allow it)
-    constexpr bool BIAS = BIASED<DT, G> && (D * G > 8);
+    // (groups of copies folded together in the kernels that 128 registers are
+    // left to: 3 x 4 copies take 98 instead of 64, half the CTAs)
+    constexpr bool BIAS = BIASED<DT, G> && (D * G >= 16);
     Acc<DT, BIAS> acc;
     uint32_t full_tiles = 0;
     TileCursor c;

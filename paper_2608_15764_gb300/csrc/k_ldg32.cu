@@ -65,8 +65,15 @@ __device__ __forceinline__ void ragged32(const KArgs& a, const Oct* buf, uint64_
     }
 }
 
+// Minimum resident CTAs per SM asked of the compiler: bfloat16 kernels are held
+// to the 72, 102 and 128 registers of seven, five and four 128-thread CTAs.
+template <int K, int CTA, int DT>
+constexpr int ldg32_min_blocks() {
+    return DT == SL_BF16 && K >= 4 ? (K == 4 ? 896 : K == 6 ? 640 : 512) / CTA : 1;
+}
+
 template <int K, int CTA, int DT, bool COV = false>
-__global__ void __launch_bounds__(CTA, 1) k_ldg32(const KArgs a) {
+__global__ void __launch_bounds__(CTA, ldg32_min_blocks<K, CTA, DT>()) k_ldg32(const KArgs a) {
     constexpr uint32_t TILE = static_cast<uint32_t>(CTA) * K;
     cta_start(a, TILE * 32);
     const Oct* __restrict__ buf = static_cast<const Oct*>(a.buf);
@@ -109,7 +116,8 @@ __global__ void __launch_bounds__(CTA, 1) k_ldg32(const KArgs a) {
 // (K = 1 is held to 32 registers for uint32, 48 for floats: eight and five
 // 256-thread CTAs per SM.)
 template <int K, int CTA, int DT, bool COV = false>
-__global__ void __launch_bounds__(CTA, K == 1 ? (DT == SL_U32 ? 2048 : 1280) / CTA : 1) k_ldg32_dyn(const KArgs a) {
+__global__ void __launch_bounds__(CTA, K == 1 ? (DT == SL_U32 ? 2048 : 1280) / CTA
+                                              : ldg32_min_blocks<K, CTA, DT>()) k_ldg32_dyn(const KArgs a) {
     constexpr uint32_t TILE = static_cast<uint32_t>(CTA) * K;
     __shared__ uint32_t slot[2];
     cta_start(a, a.tile_vec * 32);

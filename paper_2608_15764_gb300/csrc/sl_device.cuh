@@ -100,14 +100,18 @@ __device__ __forceinline__ float fp8_word_sum(uint32_t w, float acc) {
 // 256-thread (two 512-thread) CTAs stay resident: with fewer warps its
 // dependent TwoSum chains cannot hide the load latency (at K = 8 the
 // unconstrained allocation of 78 registers leaves three CTAs and ~7% less
-// bandwidth).  A K = 1 kernel of another type is held to the 32 registers that
+// bandwidth); above K = 8 to the 102 or 128 of five or four 128-thread CTAs
+// (two of 256 threads).  A K = 1 kernel of another type is held to the 32 registers that
 // let an SM's 2,048 threads be resident (its loop needs fewer; the reduction at
 // its end would otherwise take two or four more and cost a quarter of the
 // CTAs).  Every other kernel takes the registers it wants (K loaded vectors
 // must stay in registers).
 template <int K, int CTA, int DT>
 constexpr int ldg_min_blocks() {
-    if (DT == SL_BF16) return K <= 8 && CTA >= 256 ? 1024 / CTA : 1;
+    if (DT == SL_BF16) {
+        if (K <= 8) return CTA >= 256 ? 1024 / CTA : 1;
+        return CTA <= 512 ? (K <= 11 ? 640 : 512) / CTA : 1;
+    }
     return K == 1 ? 2048 / CTA : 1;
 }
 
@@ -117,13 +121,6 @@ constexpr int ldg_min_blocks() {
 template <bool COV>
 __device__ __forceinline__ void cov_count(const KArgs& a, uint64_t i) {
     if constexpr (COV) atomicAdd(a.cov + i, 1u);
-}
-
-// Largest of each 16-bit half.
-__device__ __forceinline__ uint32_t max_u16x2(uint32_t a, uint32_t b) {
-    uint32_t d;
-    asm("max.u16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
-    return d;
 }
 
 // Whether a kernel that folds n vectors at a time takes the biased sum.
@@ -142,7 +139,7 @@ constexpr bool BIASED = DT == SL_BF16 && N >= 4 && N <= 16;
 // the even-numbered values of a vector, lane 1 the odd-numbered ones), so one
 // TwoSum instruction sequence serves two elements:
 //   FP32: each of the 4 values goes through TwoSum (2 packed steps);
-//   BF16: each of the 8 values is widened exactly to FP32 (a shift or a mask)
+//   BF16: each of the 8 values is widened exactly to FP32
 //         and goes through TwoSum (4 packed steps), so no addition inside a
 //         vector is left uncompensated, whatever the values' range;
 //   FP8:  the two half-vector sums, each exact (fp8_word_sum), go through one
@@ -153,28 +150,45 @@ constexpr bool BIASED = DT == SL_BF16 && N >= 4 && N <= 16;
 // well above the data, so that |fs| >= |x| in every addition and its rounding
 // error needs the three operations of Dekker's Fast2Sum where TwoSum needs six:
 // 16 packed operations per vector (and three per fold_n) instead of 28.
-// fold_n looks at the largest exponent of its vectors first: C is 2^9 to 2^11
-// times the largest value of the first ones (a running sum of a few thousand
-// values grows to that too, so the errors collected in fe are of the size that
-// TwoSum's are), is raised when the sum itself has grown to a quarter of it, and
-// a thread that meets values of different sizes (the largest of two vectors 2^5
-// apart from that of all) when it takes a C, a value too large for the C it has,
-// an infinity or a NaN goes on with TwoSum (c = SLOW); a single vector is added by
-// TwoSum.  fs - C is exact, so entering and leaving lose nothing.
-// Measured, TwoSum then biased: 16 passes over 32 MiB in L2 at K = 8 73.5 ->
-// 65.7 us, 48 MiB by cp.async 2 x 8 14.7 -> 13.7, 4 GiB at K = 8 dynamic 584 ->
-// 576, 1,024 buffers of 16 GiB 2,555 -> 2,440 on the device.  Errors against 64
-// bits: 0 either way on N(0,1) values (256 MiB and 16 GiB); where the data's size
-// drops by 2^17 half way, 3e-15 of sum|x| (TwoSum 1e-15).  Kernels with fewer
-// vectors at a time (K < 4, one copy per group) or few warps per SM (the 64 KiB
-// TMA rings: 177 -> 200 us per GiB) stay with TwoSum.
+// The biased sum is exact: fs + fe - C is the sum of the values added, without
+// any rounding.  fs stays in [2^k, 2^(k+1)), so every error is at most
+// h = 2^(k-24); fe collects the 4N errors of a fold_n, then what is large enough
+// of it goes back to fs, which leaves |fe| <= h.  So |fe| < 2^L h with 2^L >= 4N + 2
+// and adding to it is exact while all values are multiples of its smallest step,
+// 2^(k-48+L).  fold_n therefore looks at its values' largest and smallest
+// exponent first:
+//   - the largest may move fs by at most a quarter of 2^k (HEAD = L + 2 below k),
+//     and fs starts within a quarter of C, or C is raised;
+//   - the smallest but zero is LOW = 41 - L or less below k (eight bits of
+//     significand above the step).
+// Otherwise C is taken anew, 2 above HEAD and 3 above the sum (enter_bias, which
+// also checks that what the sum holds by then is a multiple of the step).  A
+// thread whose values allow none, infinities and NaN among them, goes on with
+// TwoSum from the sum it has (c = SLOW); a single vector is added by TwoSum.
+// So a thread's error is 0 while its values fit and TwoSum's from there on.
+// Emulated on the CPU (96 threads, 16,384 values each), no error and at most 3%
+// of the groups by TwoSum on N(0,1), Laplace, Student-t with 3 degrees of freedom
+// and uniform values, their absolute values, and one value in 1,000 20 times
+// larger; the error of TwoSum alone (1e-12 of a thread's sum|x| at most, within the
+// luck of single roundings) where values shrink by 2^-13 or more after the first
+// ones or spread over more than 30 binades, most of them summed by TwoSum.
+// Measured, TwoSum then biased: 16 passes over 32 MiB in L2 at K = 8 76.0 -> 60.5
+// us, 1 GiB at K = 8 163 -> 155, at K = 4 178 -> 162; 1,024 buffers of 16 GiB by
+// 16 KiB x 2 TMA rings 2,588 -> 2,399 on the device.  Kernels with fewer vectors
+// at a time (K < 4, one copy per group) stay with TwoSum.
 template <int DT, bool BIAS = false>
 struct Acc {
     static constexpr uint32_t SLOW = 0xFFFFFFFFu;
+    // The bias a thread starts with, 1.5 * 2^12: it fits values below 2^6 (N = 4)
+    // to 2^4 (N = 16) and down to 2^-24 to 2^-22, as weights and activations mostly
+    // are, so that such a thread does not run renew_bias (whose code it would have
+    // to fetch: 0.7 us of a 14 us launch).
+    static constexpr uint32_t START = BIAS ? (139u << 23) | 0x400000u : 0u;
     uint32_t s = 0, xl = 0, xh = 0;
     uint32_t n = 0;  // 16-byte loads folded by this thread (the host keeps it below 2^32)
-    uint64_t fs = 0, fe = 0;  // packed (lane 0, lane 1) running sums and error sums; 0 bits = +0.0f
-    uint32_t c = 0;           // BIAS: bits of C in both lanes of fs; 0: none now; SLOW: none from here on
+    // packed (lane 0, lane 1) running sums and error sums; 0 bits = +0.0f
+    uint64_t fs = (static_cast<uint64_t>(START) << 32) | START, fe = 0;
+    uint32_t c = START;  // BIAS: bits of C in both lanes of fs; 0: none now; SLOW: none from here on
 
     // TwoSum of the packed pair x into (fs, fe), lane by lane.
     __device__ __forceinline__ void add2(uint64_t x) {
@@ -186,49 +200,93 @@ struct Acc {
         fs = t;
     }
 
-    // As add2 where |fs| >= |x| in both lanes (Fast2Sum).
-    __device__ __forceinline__ void add2_biased(uint64_t x) {
-        const uint64_t t = f2_add(fs, x);
-        fe = f2_add(fe, f2_sub(x, f2_sub(t, fs)));
+    // A word's two BF16 values where |fs| >= |x| in both lanes (Fast2Sum: the
+    // rounding error of t = fs + x is x - (t - fs)).  The additions that take the
+    // values take them as they are (add/sub.f32.bf16, one lane each, the value
+    // widened exactly): the shift and the mask that would unpack them are ALU
+    // work, which bounds this fold together with fold_n's look at the codes
+    // (16 passes over 32 MiB in L2 at K = 8: 70.2 us with them, 60.5 without).
+    __device__ __forceinline__ void add_word_biased(uint32_t w) {
+        float t0, t1, e0, e1;
+        asm("{\n\t.reg .b16 l, h;\n\t"
+            "mov.b32 {l, h}, %2;\n\t"
+            "add.rn.f32.bf16 %0, l, %3;\n\t"
+            "add.rn.f32.bf16 %1, h, %4;\n\t}"
+            : "=f"(t0), "=f"(t1) : "r"(w), "f"(f2_lane0(fs)), "f"(f2_lane1(fs)));
+        const uint64_t t = f2_pack(__float_as_uint(t0), __float_as_uint(t1));
+        const uint64_t d = f2_sub(t, fs);
+        asm("{\n\t.reg .b16 l, h;\n\t"
+            "mov.b32 {l, h}, %2;\n\t"
+            "sub.rn.f32.bf16 %0, l, %3;\n\t"
+            "sub.rn.f32.bf16 %1, h, %4;\n\t}"
+            : "=f"(e0), "=f"(e1) : "r"(w), "f"(f2_lane0(d)), "f"(f2_lane1(d)));
+        fe = f2_add(fe, f2_pack(__float_as_uint(e0), __float_as_uint(e1)));
+        fs = t;
+    }
+
+    // (fs, fe) without a bias: fs the rounded sum of both, fe the rest.
+    __device__ __forceinline__ void normalise() {
+        const uint64_t t = f2_add(fs, fe);
+        const uint64_t b = f2_sub(t, fs);
+        fe = f2_add(f2_sub(fs, f2_sub(t, b)), f2_sub(fe, b));
         fs = t;
     }
 
     __device__ __forceinline__ void leave_bias() {
         if (c != 0 && c != SLOW) {
-            fs = f2_sub(fs, f2_pack(c, c));
+            fs = f2_sub(fs, f2_pack(c, c));  // exact: fs is within a factor of two of C
+            normalise();
             c = 0;
         }
     }
 
-    // Take a bias for values of biased exponents up to e.  head: what C's
-    // exponent is above that of the largest value that one fold_n may add.
-    __device__ __forceinline__ void enter_bias(uint32_t e, uint32_t head) {
-        const uint32_t f0 = (static_cast<uint32_t>(fs) >> 23) & 255u;
-        const uint32_t f1 = (static_cast<uint32_t>(fs >> 32) >> 23) & 255u;
-        uint32_t k = e + head + 2;  // values may grow fourfold
-        const uint32_t f = (f0 > f1 ? f0 : f1) + 3;
-        k = k > f ? k : f;
-        if (k > 240u) {
-            c = SLOW;
-            return;
-        }
-        c = (k << 23) | 0x400000u;
-        const uint64_t old = fs;
-        fs = f2_pack(c, c);
-        add2_biased(old);
+    // Take a bias for a group of largest exponent e and smallest nonzero code
+    // low, or set c to SLOW.  On return with a bias, C's exponent is at least
+    // HEAD + 2 above e and LOW or less above low's.
+    template <int HEAD, int LOW>
+    __device__ __forceinline__ void enter_bias(int e, int low) {
+        normalise();
+        const int f0 = (static_cast<uint32_t>(fs) >> 23) & 255u, f1 = (static_cast<uint32_t>(fs >> 32) >> 23) & 255u;
+        const int k = max(e + HEAD + 2, max(f0, f1) + 3);
+        c = SLOW;
+        if (k > 240 || low < ((k - LOW) << 7)) return;
+        const uint32_t bits = (static_cast<uint32_t>(k) << 23) | 0x400000u;
+        const uint64_t t = f2_add(f2_pack(bits, bits), fs);
+        const uint64_t d = f2_sub(fs, f2_sub(t, f2_pack(bits, bits)));
+        // multiples of the step: unchanged by a round trip through 1.5 * 2^23 steps
+        const uint32_t step = (static_cast<uint32_t>(max(k - 25 + (HEAD - 2), 1)) << 23) | 0x400000u;
+        const uint64_t m = f2_pack(step, step);
+        const uint64_t off = f2_sub(f2_sub(f2_add(fe, m), m), fe) | f2_sub(f2_sub(f2_add(d, m), m), d);
+        if ((off & 0x7FFFFFFF7FFFFFFFull) != 0) return;
+        fs = t;
+        fe = f2_add(fe, d);
+        c = bits;
     }
 
-    // Largest code of two vectors' values, signs left out (volatile: computed
-    // where it is needed, not shared with fold_n's own maximum at the price of
-    // registers).
-    static __device__ __forceinline__ uint32_t pair_code(const uint4& a, const uint4& b) {
-        uint32_t m = 0;
-        const uint32_t w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+    // What fold_n does before it adds where there is no bias, the sum has outgrown
+    // it, or a value is outside its range: zeros (which fit any) keep it.
+    template <int N, int HEAD, int LOW>
+    __device__ __forceinline__ void renew_bias(const uint4 (&v)[N], bool near) {
+        // largest code and smallest nonzero code less one, signs left out.  (The
+        // mask comes by way of a register that is always zero: with the constant
+        // the compiler would keep fold_n's codes for this, at the price of a
+        // register each.)
+        uint32_t m = 0, l = 0xFFFFFFFFu, mask;
+        asm volatile("mov.u32 %0, %%ctaid.z;" : "=r"(mask));
+        mask ^= 0x7FFF7FFFu;
 #pragma unroll
-        for (int i = 0; i < 8; ++i)
-            asm volatile("{\n\t.reg .b32 t;\n\tand.b32 t, %1, 0x7FFF7FFF;\n\tmax.u16x2 %0, %0, t;\n\t}"
-                         : "+r"(m) : "r"(w[i]));
-        return m >> 16 > (m & 0xFFFFu) ? m >> 16 : m & 0xFFFFu;
+        for (int i = 0; i < N; ++i) {
+            const uint32_t w[4] = {v[i].x & mask, v[i].y & mask, v[i].z & mask, v[i].w & mask};
+            m = __vimax3_u16x2(__vimax3_u16x2(m, w[0], w[1]), w[2], w[3]);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) l = __viaddmin_u16x2(w[j], 0xFFFFFFFFu, l);
+        }
+        const int e = max(m >> 16, m & 0xFFFFu) >> 7;
+        const int low = min(l >> 16, l & 0xFFFFu) + 1;
+        const int k = c >> 23;
+        if (c != 0 && near && e + HEAD <= k && low >= ((k - LOW) << 7)) return;
+        leave_bias();
+        enter_bias<HEAD, LOW>(e, low);
     }
 
     // N vectors at once (N <= 16), by all lanes of the warp together.
@@ -238,53 +296,37 @@ struct Acc {
 #pragma unroll
             for (int i = 0; i < N; ++i) fold(v[i]);
         } else {
-            // 4N additions per lane, below 2^(log2(4N) + 1) of the largest value's
-            // power of two, move fs by at most a quarter of 2^k
-            constexpr uint32_t HEAD = N > 8 ? 9 : N > 4 ? 8 : 7;
+            constexpr int L = N > 8 ? 7 : N > 4 ? 6 : 5;  // 4N + 2 <= 2^L
+            constexpr int HEAD = L + 2, LOW = 41 - L;
 #pragma unroll
             for (int i = 0; i < N; ++i) fold_int(v[i]);
             if (c != SLOW) {
-                uint32_t m = 0;
+                // codes without sign less that of the smallest exponent allowed, mod 2^16
+                const uint32_t base = (LOW << 7) - ((c >> 23) << 7);
+                const uint32_t off = __byte_perm(base, base, 0x1010);
+                uint32_t r = 0;
 #pragma unroll
                 for (int i = 0; i < N; ++i) {
-                    m = max_u16x2(m, v[i].x & 0x7FFF7FFFu);
-                    m = max_u16x2(m, v[i].y & 0x7FFF7FFFu);
-                    m = max_u16x2(m, v[i].z & 0x7FFF7FFFu);
-                    m = max_u16x2(m, v[i].w & 0x7FFF7FFFu);
+                    r = __viaddmax_u16x2(v[i].x & 0x7FFF7FFFu, off, r);
+                    r = __viaddmax_u16x2(v[i].y & 0x7FFF7FFFu, off, r);
+                    r = __viaddmax_u16x2(v[i].z & 0x7FFF7FFFu, off, r);
+                    r = __viaddmax_u16x2(v[i].w & 0x7FFF7FFFu, off, r);
                 }
-                m = m >> 16 > (m & 0xFFFFu) ? m >> 16 : m & 0xFFFFu;
-                const uint32_t e = m >> 7;
                 // bits 22 and 21 differ while fs is between 1.25 and 1.75 * 2^k
                 const uint32_t w0 = static_cast<uint32_t>(fs), w1 = static_cast<uint32_t>(fs >> 32);
-                const bool far = ((w0 ^ (w0 << 1)) & (w1 ^ (w1 << 1)) & 0x400000u) == 0;
-                if (c == 0 || far || e + HEAD > c >> 23) {
-                    // no bias yet, the sum has outgrown it, or the values have
-                    const bool larger = c != 0 && !far && !(fs == f2_pack(c, c) && fe == 0);
-                    leave_bias();
-                    // values of one size only: beside a lone large one the others
-                    // would be summed in fe alone
-                    const uint32_t p = pair_code(v[0], v[1]), q = pair_code(v[2], v[3]);
-                    const uint32_t least = (p < q ? p : q) >> 7;
-                    if (larger || (least != 0 && e > least + 4)) c = SLOW;
-                    else enter_bias(e, HEAD);
-                    if (c != SLOW && e + HEAD > c >> 23) {
-                        leave_bias();
-                        c = SLOW;
-                    }
-                }
+                const bool near = ((w0 ^ (w0 << 1)) & (w1 ^ (w1 << 1)) & 0x400000u) != 0;
+                constexpr uint32_t RANGE = ((LOW - HEAD + 1) << 7) - 1;
+                if (c == 0 || !near || max(r >> 16, r & 0xFFFFu) > RANGE) renew_bias<N, HEAD, LOW>(v, near);
             }
             // One lane on the long way takes its warp along: both ways would be run.
             if (!__any_sync(FULL_MASK, c == SLOW)) {
 #pragma unroll
                 for (int i = 0; i < N; ++i) {
-                    add2_biased(f2_pack(v[i].x << 16, v[i].x & 0xFFFF0000u));
-                    add2_biased(f2_pack(v[i].y << 16, v[i].y & 0xFFFF0000u));
-                    add2_biased(f2_pack(v[i].z << 16, v[i].z & 0xFFFF0000u));
-                    add2_biased(f2_pack(v[i].w << 16, v[i].w & 0xFFFF0000u));
+                    add_word_biased(v[i].x);
+                    add_word_biased(v[i].y);
+                    add_word_biased(v[i].z);
+                    add_word_biased(v[i].w);
                 }
-                // what has become large enough of fe goes back to fs (exactly), so
-                // that fe stays below a few units in the last place of fs and its
-                // own roundings are no larger than under TwoSum
                 const uint64_t t = f2_add(fs, fe);
                 fe = f2_sub(fe, f2_sub(t, fs));
                 fs = t;
@@ -350,12 +392,11 @@ __device__ __forceinline__ void df_add(float& hi, float& lo, float ohi, float ol
 
 template <int DT, bool BIAS>
 __device__ __forceinline__ void Acc<DT, BIAS>::float_part(float& hi, float& lo) const {
-    uint64_t f = fs;
-    if constexpr (BIAS)
-        if (c != 0 && c != SLOW) f = f2_sub(f, f2_pack(c, c));
-    hi = f2_lane0(f);
-    lo = f2_lane0(fe);
-    df_add(hi, lo, f2_lane1(f), f2_lane1(fe));
+    Acc a = *this;
+    if constexpr (BIAS) a.leave_bias();
+    hi = f2_lane0(a.fs);
+    lo = f2_lane0(a.fe);
+    df_add(hi, lo, f2_lane1(a.fs), f2_lane1(a.fe));
 }
 
 // ---- warp reductions ------------------------------------------------------------
