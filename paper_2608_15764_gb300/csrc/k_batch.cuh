@@ -73,6 +73,26 @@ __device__ __forceinline__ WarpPartial warp_partial(const Acc<DT, BIAS>& acc) {
 // thread 0 writes index j + 3, so there are four index words (with three,
 // index j + 3 would be index j's); they read descriptor j + 1 and partials j
 // while descriptor j + 2 and partials j + 1 are written: two of each.
+// The thread's place is read by hand where it is used: the compiler would keep
+// what it computes from threadIdx (addresses, lane, warp, comparisons) in
+// registers through stream(), ten of them in an LDG kernel (K = 4 uint32 42 -> 33
+// registers, K = 16 102 -> 81).
+__device__ __forceinline__ uint32_t tid_here() {
+    uint32_t t;
+    asm volatile("mov.u32 %0, %%tid.x;" : "=r"(t));
+    return t;
+}
+__device__ __forceinline__ uint32_t threads_here() {
+    uint32_t t;
+    asm volatile("mov.u32 %0, %%ntid.x;" : "=r"(t));
+    return t;
+}
+__device__ __forceinline__ uint32_t grid_here() {
+    uint32_t t;
+    asm volatile("mov.u32 %0, %%nctaid.x;" : "=r"(t));
+    return t;
+}
+
 template <bool FLOATS, typename Stream>
 __device__ __forceinline__ void batch_items(const BArgs& a, Stream stream) {
     __shared__ BatchItem slot[2];
@@ -88,25 +108,23 @@ __device__ __forceinline__ void batch_items(const BArgs& a, Stream stream) {
     for (uint32_t j = 0;; ++j) {
         // sidx[j & 3]: this item, [(j + 1) & 3]: the next, [(j + 2) & 3]: being claimed
         uint32_t claim = 0xFFFFFFFFu;
-        if (threadIdx.x == 0) {
+        if (tid_here() == 0) {
             const uint32_t ahead = vidx[(j + 1) & 3];
             if (ahead < a.nitems) {
                 asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(&slot[(j + 1) & 1])),
                              "l"(a.items + ahead) : "memory");
-                claim = 2 * gridDim.x + atomicAdd(a.next, 1u);
+                claim = 2 * grid_here() + atomicAdd(a.next, 1u);
             }
         }
-        {
-            const WarpPartial w = stream(it);
-            if ((threadIdx.x & 31) == 0) wp[j & 1][threadIdx.x >> 5] = w;
-        }
-        if (threadIdx.x == 0) {
+        const WarpPartial mine = stream(it);
+        const uint32_t tid = tid_here(), warp = tid >> 5, lane = tid & 31, nw = threads_here() >> 5;
+        if (lane == 0) wp[j & 1][warp] = mine;
+        if (tid == 0) {
             asm volatile("cp.async.wait_all;" ::: "memory");
             vidx[(j + 2) & 3] = claim;
         }
         __syncthreads();
         const uint32_t cur = vidx[j & 3], next = vidx[(j + 1) & 3];
-        const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
         if (warp == j % nw) {
             uint32_t s = 0;
             uint64_t x = 0, n = 0;
@@ -143,7 +161,7 @@ __device__ __forceinline__ WarpPartial ldg_item(const BatchItem& it) {
     constexpr uint32_t TILE = static_cast<uint32_t>(CTA) * K;
     Acc<DT, BIASED<DT, K>> acc;
     const uint32_t nfull = it.nvec / TILE;
-    const uint4* p = it.ptr + threadIdx.x;
+    const uint4* p = it.ptr + tid_here();
 #pragma unroll 1
     for (uint32_t t = 0; t < nfull; ++t, p += TILE) {
         uint4 v[K];
@@ -154,15 +172,16 @@ __device__ __forceinline__ WarpPartial ldg_item(const BatchItem& it) {
     acc.n = nfull * K;
     const uint32_t rem = it.nvec - nfull * TILE;
     if (rem) {
+        const uint32_t tid = tid_here();
         uint4 v[K];
 #pragma unroll
         for (int k = 0; k < K; ++k) {
-            if (threadIdx.x + k * CTA < rem) v[k] = ldg16<SL_COP_CG>(p + k * CTA);
+            if (tid + k * CTA < rem) v[k] = ldg16<SL_COP_CG>(p + k * CTA);
             else v[k] = make_uint4(0u, 0u, 0u, 0u);
         }
 #pragma unroll
         for (int k = 0; k < K; ++k) {
-            if (threadIdx.x + k * CTA < rem) {
+            if (tid + k * CTA < rem) {
                 acc.fold(v[k]);
                 acc.n += 1;
             }
@@ -171,8 +190,21 @@ __device__ __forceinline__ WarpPartial ldg_item(const BatchItem& it) {
     return warp_partial(acc);
 }
 
+// Minimum resident CTAs per SM asked of the compiler: what 5K + 12 registers
+// (uint32) or 5K + 32 (floats) allow, the K loaded vectors, the sums and the
+// fold's temporaries.  Left to itself it takes more where a CTA is lost by it (1,024
+// buffers of 16 GiB: FP32 K = 6 at 512 threads 70 registers, one CTA per SM, 2,710
+// us; 58, two, 2,330) or fewer than the loads in flight need.
 template <int K, int CTA, int DT>
-__global__ void __launch_bounds__(CTA, DT == SL_BF16 ? ldg_min_blocks<K, CTA, DT>() : 1) kb_ldg(const BArgs a) {
+constexpr int kb_ldg_min_blocks() {
+    int regs = DT == SL_U32 || (DT == SL_FP8_E4M3 && K == 1) ? 5 * K + 12 : K <= 2 ? 40 : 5 * K + 32;
+    if (DT == SL_BF16 && K == 8) regs = CTA >= 256 ? 64 : 80;
+    regs = regs < 32 ? 32 : regs > 128 ? 128 : (regs + 7) / 8 * 8;
+    return 65536 / (CTA * regs) > 0 ? 65536 / (CTA * regs) : 1;
+}
+
+template <int K, int CTA, int DT>
+__global__ void __launch_bounds__(CTA, kb_ldg_min_blocks<K, CTA, DT>()) kb_ldg(const BArgs a) {
     batch_items<DT != SL_U32>(a, [](const BatchItem& it) { return ldg_item<K, CTA, DT>(it); });
 }
 

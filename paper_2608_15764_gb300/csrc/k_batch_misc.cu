@@ -16,35 +16,46 @@ __device__ __forceinline__ void kb_cp_wait() { asm volatile("cp.async.wait_group
 // [j*cta, (j+1)*cta); each thread copies its 16 bytes of chunk j into ring
 // slot j mod D with D commit groups in flight, reads its own slot back and
 // folds (as k_cpasync).  The pipeline drains at the end of each item.
+//
+// Registers: an SM's CTAs hide each other's latency, so the budget is that of the
+// loop (32 let all 2,048 threads be resident), more where the fold would be
+// squeezed into a serial chain: 1,024 buffers of 16 GiB at 256 threads, uint32 D = 6
+// 48 -> 32 registers 2,350 -> 2,287 us; bfloat16 D = 2 32 -> 40 registers
+// 3,021 -> 2,726, but D = 1 32 -> 40 2,946 -> 3,214; FP32 D = 2 2,343 -> 2,327 (2
+// GiB: 324 -> 310).  (D and the block size are the caller's, so the cap is on
+// registers, not on CTAs per SM.)
+constexpr int kb_cpasync_regs(int d, int dt) {
+    if (dt == SL_U32 || d == 1) return 32;
+    if (dt == SL_FP8_E4M3) return d <= 4 ? 32 : 40;
+    if (dt == SL_F32) return d == 3 || d == 4 ? 32 : d <= 5 ? 40 : 48;
+    return d <= 5 ? 40 : 48;
+}
+
 template <int D, int DT>
-__global__ void __launch_bounds__(1024) kb_cpasync(const BArgs a) {
+__global__ void __maxnreg__(kb_cpasync_regs(D, DT)) kb_cpasync(const BArgs a) {
     extern __shared__ __align__(128) uint4 cp_ring[];  // [D][cta], 128-byte aligned (cp.async destinations)
-    const uint32_t cta = blockDim.x, t = threadIdx.x;
-    const uint32_t my0 = smem_addr(cp_ring + t), stride = cta * 16u;
     batch_items<DT != SL_U32>(a, [&](const BatchItem& it) {
+        const uint32_t cta = blockDim.x, t = tid_here();
+        const uint32_t my0 = smem_addr(cp_ring) + t * 16u, stride = cta * 16u;
         Acc<DT> acc;
-        const uint32_t nchunks = (it.nvec + cta - 1) / cta;
-        uint32_t islot = 0, cslot = 0;
 #pragma unroll
         for (int g = 0; g < D - 1; ++g) {
             const uint32_t v = static_cast<uint32_t>(g) * cta + t;
-            if (static_cast<uint32_t>(g) < nchunks && v < it.nvec) kb_cp_async16(my0 + islot * stride, it.ptr + v);
+            if (v < it.nvec) kb_cp_async16(my0 + g * stride, it.ptr + v);
             kb_cp_commit();
-            islot = (islot + 1 == D) ? 0 : islot + 1;
         }
+        uint32_t slot = 0;
 #pragma unroll 1
-        for (uint32_t j = 0; j < nchunks; ++j) {
-            const uint32_t g = j + D - 1;
-            const uint32_t v = g * cta + t;
-            if (g < nchunks && v < it.nvec) kb_cp_async16(my0 + islot * stride, it.ptr + v);
+        for (uint32_t base = 0; base < it.nvec; base += cta) {
+            const uint32_t v = base + t, ahead = v + (D - 1) * cta;
+            if (ahead < it.nvec) kb_cp_async16(my0 + (slot == 0 ? D - 1 : slot - 1) * stride, it.ptr + ahead);
             kb_cp_commit();
-            islot = (islot + 1 == D) ? 0 : islot + 1;
             kb_cp_wait<D - 1>();
-            if (j * cta + t < it.nvec) {
-                acc.fold(lds16(my0 + cslot * stride));
+            if (v < it.nvec) {
+                acc.fold(lds16(my0 + slot * stride));
                 acc.n += 1;
             }
-            cslot = (cslot + 1 == D) ? 0 : cslot + 1;
+            slot = (slot + 1 == D) ? 0 : slot + 1;
         }
         kb_cp_wait<0>();
         return warp_partial(acc);
