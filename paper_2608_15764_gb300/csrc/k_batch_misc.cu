@@ -105,23 +105,21 @@ __global__ void __launch_bounds__(1024) kb_tma(const BArgs a) {
         if (lane == 0) {
             uint32_t armed = 0, last_par = 0, s = 0, r = 0;
             bool stop = false;
-            // `item` streams while the descriptor of the next one is on its
-            // way and the one after it is being claimed
-            uint32_t item = blockIdx.x, ahead = blockIdx.x + gridDim.x;
+            // The next item is claimed, and its descriptor fetched, when no more
+            // stages are left to issue than are in flight: claimed any earlier, items
+            // are dealt out before it shows which CTAs are fast.
+            uint32_t item = blockIdx.x;
             BatchItem it = a.items[item];  // the host launches at most nitems CTAs
             while (!stop) {
                 const bool done = item >= a.nitems;
                 uint32_t nstage = 1, nbytes = 0;
-                BatchItem it1{nullptr, 0u, 0u};
-                uint32_t claim = 0xFFFFFFFFu;
                 if (!done) {
                     nbytes = it.nvec * 16u;
                     nstage = (nbytes + S - 1) / S;
-                    if (ahead < a.nitems) {
-                        it1 = a.items[ahead];
-                        claim = 2 * gridDim.x + atomicAdd(a.next, 1u);
-                    }
                 }
+                const uint32_t ask = nstage > nst ? nstage - nst : 0;
+                uint32_t next = 0xFFFFFFFFu;
+                BatchItem it1{nullptr, 0u, 0u};
                 for (uint32_t k = 0; k < nstage; ++k) {
                     if (r > 0 && !bounded_wait(empty0 + 8 * s, (r - 1) & 1u, a.err, a.timeout_ns, &abort_flag, true,
                                                DEV_ERR_TIMEOUT_EMPTY)) {
@@ -145,11 +143,14 @@ __global__ void __launch_bounds__(1024) kb_tma(const BArgs a) {
                         last_par = (last_par & ~(1u << s)) | ((r & 1u) << s);
                     }
                     if (++s == nst) { s = 0; ++r; }
+                    if (k == ask && !done) {
+                        next = gridDim.x + atomicAdd(a.next, 1u);
+                        if (next < a.nitems) it1 = a.items[next];
+                    }
                 }
                 if (done) stop = true;
-                item = ahead;
+                item = next;
                 it = it1;
-                ahead = claim;
             }
             for (uint32_t q = 0; q < nst; ++q)
                 if (armed & (1u << q))
