@@ -20,7 +20,7 @@ namespace sl {
 const void* batch_ldg_kernel(int dtype, int k, int cta);
 const void* batch_ldg_any_kernel(int k, int cta);
 const void* batch_cpasync_kernel(int dtype, int d);
-const void* batch_tma_kernel(int dtype, int batch, bool small_ring);
+const void* batch_tma_kernel(int dtype, int batch, bool biased);
 cudaError_t launch_batch_combine(const BufSeg* segs, uint32_t nbuf, const WarpPartial* parts, uint32_t* err,
                                  uint32_t* next, uint32_t nclasses, sl_result* out, uint32_t* host_err,
                                  cudaStream_t s);
@@ -129,6 +129,19 @@ int plan_ctas(const void* fn, const Group& g, int sms, int* ctas) {
     return SL_OK;
 }
 
+// Whether a TMA class of bfloat16 buffers takes the biased sum: its serial chain
+// is longer than TwoSum's, so it pays where the rings leave room for 24 consumer
+// warps per SM (1,024 buffers of 16 GiB, TwoSum then biased: 16 KiB x 4 at 256
+// threads, 24 warps, 2,561 -> 2,415 us on the device; 16 KiB x 2 at 128 threads, 28 warps,
+// 2,465 -> 2,295; 16 KiB x 4 at 128 threads, 12 warps, 2,538 -> 2,546; 16 KiB x 5 at 256, 16 warps,
+// 2,717 -> 2,724; 64 KiB x 2 at 256, 8 warps, 2,744 -> 3,122), and where a stage is
+// whole groups of four vectors per thread, since every single vector drops
+// the bias (16 KiB x 4 at 192 threads: 2,874 -> 3,659).
+bool tma_biased(const sl_config& c, int smem_optin) {
+    const int64_t ring = static_cast<int64_t>(c.stages) * c.stage_bytes;
+    return smem_optin / ring * (c.cta / 32) >= 24 && c.stage_bytes / 16 % (4 * c.cta) == 0;
+}
+
 // Kernel, block shape, shared memory and persistent grid of one group.
 int plan_group(Group& g, int sms, int smem_optin) {
     const sl_config& c = g.cfg;
@@ -164,8 +177,7 @@ int plan_group(Group& g, int sms, int smem_optin) {
                          "(tma_ring must be SL_RING_CTA)");
         // consumer threads read their last 4 vectors of a stage (1 where they
         // read fewer) into registers before releasing it
-        g.fn = sl::batch_tma_kernel(g.dtype, c.stage_bytes / 16 >= 4 * c.cta ? 4 : 1,
-                                    static_cast<int64_t>(c.stages) * c.stage_bytes <= (56 << 10));
+        g.fn = sl::batch_tma_kernel(g.dtype, c.stage_bytes / 16 >= 4 * c.cta ? 4 : 1, tma_biased(c, smem_optin));
         g.block = c.cta + 32;
         g.smem = static_cast<size_t>(c.stages) * c.stage_bytes;
         g.slots = c.cta / 32;

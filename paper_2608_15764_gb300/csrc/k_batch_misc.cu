@@ -334,10 +334,10 @@ static const void* kb_tma_b(int dtype) {
     }
 }
 
-const void* batch_tma_kernel(int dtype, int batch, bool small_ring) {
+const void* batch_tma_kernel(int dtype, int batch, bool biased) {
     if (batch == 4)
-        return dtype == SL_BF16 && small_ring ? reinterpret_cast<const void*>(&kb_tma<SL_BF16, 4, true>)
-                                              : kb_tma_b<4>(dtype);
+        return dtype == SL_BF16 && biased ? reinterpret_cast<const void*>(&kb_tma<SL_BF16, 4, true>)
+                                          : kb_tma_b<4>(dtype);
     if (batch == 1) return kb_tma_b<1>(dtype);
     return nullptr;
 }
