@@ -113,18 +113,32 @@ void release(sl_batch* b) {
     delete b;
 }
 
-// Persistent CTAs of kernel fn at group g's block shape.
-int plan_ctas(const void* fn, const Group& g, int sms, int* ctas) {
+// Persistent CTAs of kernel fn at group g's block shape; on failure the status,
+// and what failed in *why.
+int plan_ctas(const void* fn, const Group& g, int sms, int* ctas, const char** why) {
+    int status = SL_OK;
+    const auto cuda_ok = [&](cudaError_t e, const char* what) {
+        if (e == cudaSuccess) return true;
+        (void)cudaGetLastError();
+        status = e == cudaErrorMemoryAllocation ? SL_ERR_OOM : SL_ERR_CUDA;
+        *why = what;
+        return false;
+    };
+    const auto infeasible = [&](const char* what) {
+        *why = what;
+        return SL_ERR_INFEASIBLE;
+    };
     cudaFuncAttributes fa;
-    B_TRY(cudaFuncGetAttributes(&fa, fn), "cudaFuncGetAttributes failed");
-    if (fa.localSizeBytes > 0) return bfail(SL_ERR_INFEASIBLE, "tuning entry: kernel spills registers");
-    if (g.block > fa.maxThreadsPerBlock) return bfail(SL_ERR_INFEASIBLE, "tuning entry: too many threads for this kernel");
-    if (g.smem > 0)
-        B_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(g.smem)),
-              "cudaFuncSetAttribute failed");
+    if (!cuda_ok(cudaFuncGetAttributes(&fa, fn), "cudaFuncGetAttributes failed")) return status;
+    if (fa.localSizeBytes > 0) return infeasible("tuning entry: kernel spills registers");
+    if (g.block > fa.maxThreadsPerBlock) return infeasible("tuning entry: too many threads for this kernel");
+    if (g.smem > 0 && !cuda_ok(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                    static_cast<int>(g.smem)), "cudaFuncSetAttribute failed"))
+        return status;
     int res = 0;
-    B_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&res, fn, g.block, g.smem), "occupancy query failed");
-    if (res < 1) return bfail(SL_ERR_INFEASIBLE, "tuning entry: zero occupancy");
+    if (!cuda_ok(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&res, fn, g.block, g.smem), "occupancy query failed"))
+        return status;
+    if (res < 1) return infeasible("tuning entry: zero occupancy");
     *ctas = g.cfg.grid > 0 ? g.cfg.grid : res * sms;
     return SL_OK;
 }
@@ -187,7 +201,9 @@ int plan_group(Group& g, int sms, int smem_optin) {
         return bfail(SL_ERR_ARG, "tuning entry: bad mech");
     }
     if (g.smem > static_cast<size_t>(smem_optin)) return bfail(SL_ERR_INFEASIBLE, "tuning entry: shared memory over the limit");
-    return plan_ctas(g.fn, g, sms, &g.ctas);
+    const char* why = "";
+    const int rc = plan_ctas(g.fn, g, sms, &g.ctas, &why);
+    return rc ? bfail(rc, why) : SL_OK;
 }
 
 // Bytes of a group's work items, a multiple of its unit (a tile, a ring of
@@ -217,14 +233,16 @@ uint64_t item_bytes(const Group& g) {
 // classes want the registers (CTAs per SM) of their own type's kernel.  (64
 // buffers, 16 MiB, four types in two size classes: 19.6 -> 14.0 us on the device,
 // 36 -> 29 per call.)
-int plan_units(const std::vector<Group>& groups, int sms, std::vector<Unit>* units) {
+std::vector<Unit> plan_units(const std::vector<Group>& groups, int sms) {
+    std::vector<Unit> units;
     std::vector<bool> taken(groups.size(), false);
     for (size_t i = 0; i < groups.size(); ++i) {
         if (taken[i] || groups[i].items.empty()) continue;
         Unit u;
         if (groups[i].cfg.mech == SL_LDG) {
             const void* any = sl::batch_ldg_any_kernel(groups[i].cfg.k, groups[i].cfg.cta);
-            if (any && plan_ctas(any, groups[i], sms, &u.ctas) == SL_OK) {
+            const char* why = "";  // (not reported: the group has its own kernel)
+            if (any && plan_ctas(any, groups[i], sms, &u.ctas, &why) == SL_OK) {
                 for (size_t j = i; j < groups.size(); ++j)
                     if (groups[j].entry == groups[i].entry && !groups[j].items.empty()) {
                         u.groups.push_back(static_cast<int>(j));
@@ -240,9 +258,9 @@ int plan_units(const std::vector<Group>& groups, int sms, std::vector<Unit>* uni
             u.nitems = groups[i].items.size();
         }
         for (int j : u.groups) taken[j] = true;
-        units->push_back(u);
+        units.push_back(u);
     }
-    return SL_OK;
+    return units;
 }
 
 // Everything after the argument checks; the caller releases b on failure.
@@ -295,9 +313,7 @@ int build_batch(sl_batch* b, const sl_batch_desc* descs, int32_t n, const sl_tun
     }
     std::vector<BatchItem> all;
     uint64_t slots = 0;
-    std::vector<Unit> units;
-    const int prc = plan_units(b->groups, sms, &units);
-    if (prc) return prc;
+    std::vector<Unit> units = plan_units(b->groups, sms);
     for (Unit& u : units) {
         u.item_off = all.size();
         u.part_off = slots;
