@@ -257,9 +257,15 @@ uint64_t dyn_chunk_tiles(uint64_t tiles, uint64_t tile_bytes, uint64_t grid, uin
 // cp.async 2 x 8 enqueued back to back 16.0 -> 14.5 us (16 KiB: 15.3), 96 MiB of
 // FP8 by TMA 20.6 -> 19.3, 64 MiB at K = 8 15.5 -> 14.6; dynamic chunks of plain
 // loads take 16 KiB (256 MiB 41.7 -> 41.0, 96 MiB 19.7 -> 19.1; 19.5 with 32).
-// Grid-stride plain loads with small tiles do without: 64 MiB at K = 4 took 15.4
-// us with 16 KiB and 15.1 without, 1 GiB at K = 2 177 and 173.  So do several
-// passes in one launch, which want their CTAs spread evenly (cta_finish).
+// Grid-stride launches with smaller tiles do without, since a launch that prefetches
+// lets the next one's CTAs in beside its own last ones, unevenly (cta_finish):
+// 64 MiB at K = 4 took 15.4 us with 16 KiB and 15.1 without, 1 GiB at K = 2 177 and
+// 173; 1 GiB by cp.async D = 4 at 256 threads (16 KiB) 160.5 and 151.8, D = 5 161 and
+// 151.7, D = 6 158 and 154, D = 4 of bfloat16 at 128 threads 211 and 180 (D = 8, 32 KiB: the
+// same at 1 GiB, 48 MiB 11.9 and 12.9; D = 5 of FP32 there 12.2 and 13.4).  Under
+// dynamic chunks tiles of 16 KiB still gain (48 MiB, D = 4: 12.7 and 13.1), those
+// of 8 KiB lose (bfloat16 D = 2 17.4 and 16.7).  So do several passes in one
+// launch, which want their CTAs spread evenly.
 uint32_t first_bytes(const sl_config* cfg, uint64_t tile_bytes) {
     if (cfg->passes > 1) return 0;
     switch (cfg->mech) {
@@ -268,7 +274,9 @@ uint32_t first_bytes(const sl_config* cfg, uint64_t tile_bytes) {
         if (cfg->target_loads) return 0;
         if (cfg->order == SL_DYN) return 16u << 10;
         return tile_bytes >= 32u << 10 ? 32u << 10 : 0;
-    case SL_CPASYNC: return static_cast<uint32_t>(std::min<uint64_t>(tile_bytes, 32u << 10));
+    case SL_CPASYNC:
+        if (tile_bytes < (cfg->order == SL_DYN ? 16u << 10 : 32u << 10)) return 0;
+        return static_cast<uint32_t>(std::min<uint64_t>(tile_bytes, 32u << 10));
     case SL_TMA: return cfg->tma_ring == SL_RING_CTA ? 32u << 10 : 0;
     default: return 0;
     }
