@@ -184,7 +184,9 @@ typedef struct sl_result {
     uint64_t device_ns;       /* CUDA-event time of the load kernel (sl_run);
                                  of the whole call (sl_run_host); 0 (sl_enqueue) */
     uint64_t window_ns;       /* %globaltimer: first CTA start to last CTA end (CTAs
-                                 with at least one tile) */
+                                 with at least one tile).  sl_enqueue: from the
+                                 first read, which may be a prefetch while the
+                                 kernel before it on the stream ends */
     double   fsum;            /* float dtypes: sum of the decoded payload */
     float    fsum_hi;         /* fsum as a float pair: hi = fl(fsum) */
     float    fsum_lo;         /*                       lo = fl(fsum - hi) */

@@ -786,7 +786,9 @@ int sl_enqueue_steps(const void* const* dev_bufs, int32_t nbufs, uint64_t bytes,
         q.args.done = sl::ctrl_done(c->err);
         q.args.next = dyn ? c->step_next + slot : nullptr;
         q.args.result = dev_out + i;
-        q.args.overlap = 1;  // pass 0, an ordinary launch, too: it lets pass 1 begin at its start
+        // pass 0, an ordinary launch, too lets the next one begin at its start;
+        // the last pass lets nothing begin that would wait for all of it
+        q.args.overlap = i + 1 < steps ? 1 : 2;
         rc = launch(q, s, i > 0 && !(dyn && slot == 0) ? LAUNCH_OVERLAP : LAUNCH_PLAIN);
         if (rc) return rc;
     }

@@ -73,15 +73,9 @@ __device__ __forceinline__ WarpPartial warp_partial(const Acc<DT, BIAS>& acc) {
 // thread 0 writes index j + 3, so there are four index words (with three,
 // index j + 3 would be index j's); they read descriptor j + 1 and partials j
 // while descriptor j + 2 and partials j + 1 are written: two of each.
-// The thread's place is read by hand where it is used: the compiler would keep
-// what it computes from threadIdx (addresses, lane, warp, comparisons) in
-// registers through stream(), ten of them in an LDG kernel (K = 4 uint32 42 -> 33
-// registers, K = 16 102 -> 81).
-__device__ __forceinline__ uint32_t tid_here() {
-    uint32_t t;
-    asm volatile("mov.u32 %0, %%tid.x;" : "=r"(t));
-    return t;
-}
+// What is computed from the thread's place is kept out of the registers through
+// stream() (tid_here; the same for the block's and the grid's size): ten registers
+// in an LDG kernel (K = 4 uint32 42 -> 33, K = 16 102 -> 81).
 __device__ __forceinline__ uint32_t threads_here() {
     uint32_t t;
     asm volatile("mov.u32 %0, %%ntid.x;" : "=r"(t));

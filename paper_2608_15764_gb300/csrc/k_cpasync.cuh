@@ -99,8 +99,9 @@ __global__ void __launch_bounds__(D * G > 8 ? 512 : 1024) k_cpasync(const KArgs 
             ++full_tiles;
             continue;
         }
-        const uint64_t cbase = static_cast<uint64_t>(cur) * tile_vec + threadIdx.x;
-        const uint64_t nbase = has_next ? static_cast<uint64_t>(c.tile(a)) * tile_vec + threadIdx.x : nvec;
+        const uint32_t tid = tid_here();
+        const uint64_t cbase = static_cast<uint64_t>(cur) * tile_vec + tid;
+        const uint64_t nbase = has_next ? static_cast<uint64_t>(c.tile(a)) * tile_vec + tid : nvec;
         // vectors left from this thread's first copy of the current / next
         // tile, clamped to 32 bits: copy j is in range iff j*cta < rem
         const uint32_t crem = cbase < nvec ? static_cast<uint32_t>(min(nvec - cbase, static_cast<uint64_t>(0xFFFFFFFFu))) : 0u;

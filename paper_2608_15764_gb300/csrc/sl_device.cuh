@@ -18,6 +18,15 @@ __device__ __forceinline__ uint64_t gtimer() {
     return t;
 }
 
+// threadIdx.x, read by hand where it is used: the compiler would keep what it
+// computes from threadIdx (addresses, lane, warp, comparisons) in registers
+// through the loops between.
+__device__ __forceinline__ uint32_t tid_here() {
+    uint32_t t;
+    asm volatile("mov.u32 %0, %%tid.x;" : "=r"(t));
+    return t;
+}
+
 // One 16-byte global load (paper §3: one ld.global per offered load; §4.2
 // primary cell uses .cg, which caches in L2 only).  volatile keeps every load
 // in the program and in source order.
@@ -657,7 +666,8 @@ __device__ __forceinline__ uint32_t dyn_claim(const KArgs& a) { return gridDim.x
 // begin.  In that order, so that a dependent launch never starts before everything
 // ahead of this one is complete, as if this launch had been an ordinary one.
 // A pass with a.overlap set (sl_enqueue_steps, whose buffers are only read)
-// lets the next launch begin and streams at once, and waits in cta_finish.
+// lets the next launch begin (1; the last pass, 2, does not: what follows it
+// would only wait) and streams at once, and waits in cta_finish.
 // A CTA that the launch has no tile for (index a.active or more) exits at once,
 // so that a small launch does not wait for hundreds of empty partials (64 KiB,
 // 8 CTAs of 608 with work: 6.2 -> 4.7 us).  Thread 0 keeps this CTA's
@@ -668,7 +678,8 @@ __device__ __forceinline__ uint32_t dyn_claim(const KArgs& a) { return gridDim.x
 // read first, before it waits: its CTAs are resident during the last few
 // microseconds of the kernel before it, when DRAM is nearly idle.  (A prefetch
 // returns no data and L2 is where that kernel's writes go, so the loads after
-// the wait see them.)  tile_bytes: bytes of one of the launch's tiles (chunks
+// the wait see them.)  The start stamp is taken before the first of these reads,
+// so that the window covers all that the launch reads.  tile_bytes: bytes of one of the launch's tiles (chunks
 // for SL_DYN); PF false leaves this out.
 template <bool PF = true>
 __device__ __forceinline__ void cta_start(const KArgs& a, uint32_t tile_bytes = 0) {
@@ -677,6 +688,7 @@ __device__ __forceinline__ void cta_start(const KArgs& a, uint32_t tile_bytes = 
                  "setp.ge.u32 p, b, %0;\n\t"
                  "@p exit;\n\t}" ::"r"(a.active) : "memory");
     if (PF && a.prefetch && threadIdx.x == 0) {
+        cta_start_stamp() = gtimer();
         const uint32_t ntiles = static_cast<uint32_t>(a.ntiles);
         const uint32_t part = tile_bytes < a.prefetch ? tile_bytes : a.prefetch;
         uint32_t it = blockIdx.x;
@@ -688,11 +700,12 @@ __device__ __forceinline__ void cta_start(const KArgs& a, uint32_t tile_bytes = 
                          : "memory");
         }
     }
-    asm volatile("{\n\t.reg .pred p;\n\t"
+    asm volatile("{\n\t.reg .pred p, q;\n\t"
                  "setp.eq.s32 p, %0, 0;\n\t"
+                 "setp.eq.s32 q, %0, 1;\n\t"
                  "@p griddepcontrol.wait;\n\t"
-                 "@!p griddepcontrol.launch_dependents;\n\t}" ::"r"(a.overlap) : "memory");
-    if (threadIdx.x == 0) cta_start_stamp() = gtimer();
+                 "@q griddepcontrol.launch_dependents;\n\t}" ::"r"(a.overlap) : "memory");
+    if ((threadIdx.x | (PF ? a.prefetch : 0u)) == 0) cta_start_stamp() = gtimer();
 }
 
 }  // namespace sl

@@ -37,7 +37,8 @@ struct KArgs {
     int32_t debug;          // SL_DEBUG_* flags
     int32_t overlap;        // 1: the launch streams at once and lets the next one
                             // begin (passes over buffers that are only read);
-                            // 0: it waits for the kernel before it first
+                            // 2: it streams at once; 0: it waits for the kernel
+                            // before it first
     WarpPartial* parts;     // [grid]: one partial per CTA
     uint64_t* window;       // [2]: earliest CTA start, latest CTA end
                             // (%globaltimer; ~0 and 0 before the launch)
