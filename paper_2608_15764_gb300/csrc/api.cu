@@ -252,22 +252,26 @@ uint64_t dyn_chunk_tiles(uint64_t tiles, uint64_t tile_bytes, uint64_t grid, uin
 }
 
 // Bytes that each CTA of a dependent launch prefetches into L2 (tile_bytes: one
-// tile of the configuration).  Where a CTA starts with 32 KiB or more in flight
+// tile of the configuration; room: an SM can hold more CTAs than the launch has
+// for it).  Where a CTA starts with 32 KiB or more in flight
 // (cp.async and TMA rings, large tiles) 32 KiB pay: 48 MiB of bfloat16 by
 // cp.async 2 x 8 enqueued back to back 16.0 -> 14.5 us (16 KiB: 15.3), 96 MiB of
 // FP8 by TMA 20.6 -> 19.3, 64 MiB at K = 8 15.5 -> 14.6; dynamic chunks of plain
 // loads take 16 KiB (256 MiB 41.7 -> 41.0, 96 MiB 19.7 -> 19.1; 19.5 with 32).
-// Grid-stride launches with smaller tiles do without, since a launch that prefetches
-// lets the next one's CTAs in beside its own last ones, unevenly (cta_finish):
-// 64 MiB at K = 4 took 15.4 us with 16 KiB and 15.1 without, 1 GiB at K = 2 177 and
-// 173; 1 GiB by cp.async D = 4 at 256 threads (16 KiB) 160.5 and 151.8, D = 5 161 and
-// 151.7, D = 6 158 and 154, D = 4 of bfloat16 at 128 threads 211 and 180 (D = 8, 32 KiB: the
-// same at 1 GiB, 48 MiB 11.9 and 12.9; D = 5 of FP32 there 12.2 and 13.4).  Under
-// dynamic chunks tiles of 16 KiB still gain (48 MiB, D = 4: 12.7 and 13.1), those
-// of 8 KiB lose (bfloat16 D = 2 17.4 and 16.7).  So do several passes in one
-// launch, which want their CTAs spread evenly.
-uint32_t first_bytes(const sl_config* cfg, uint64_t tile_bytes) {
-    if (cfg->passes > 1) return 0;
+// A launch that prefetches lets the next one's CTAs in beside its own last ones
+// (cta_finish).  Where an SM has room for them they land unevenly, and a
+// grid-stride launch runs as long as its fullest SM: 1 GiB by cp.async at 256
+// threads, D = 4 (uint32, eight CTAs fit, four launched) 160.5 us with a prefetch
+// and 151.8 without, D = 5 161 / 152, D = 6 158 / 154, bfloat16 D = 4 at 128 threads
+// 211 / 180.  Where the launch fills the SMs they come in as the others leave, and
+// it pays: FP32 D = 5 (four CTAs) 48 MiB 12.2 / 13.4, D = 4 at 512 threads 12.0 /
+// 13.3.  Dynamic chunks even it out: D = 4 12.7 / 13.1.  Smaller tiles do without:
+// 64 MiB of plain loads at K = 4 took 15.4 us with 16 KiB and 15.1 without, 1
+// GiB at K = 2 177 and 173, bfloat16 by cp.async D = 2 under dynamic chunks (8
+// KiB) 17.4 and 16.7.  So do several passes in one launch, which want their CTAs
+// spread evenly.
+uint32_t first_bytes(const sl_config* cfg, uint64_t tile_bytes, bool room) {
+    if (cfg->passes > 1 || (room && cfg->order != SL_DYN)) return 0;
     switch (cfg->mech) {
     case SL_LDG:
     case SL_LDG32:
@@ -275,8 +279,7 @@ uint32_t first_bytes(const sl_config* cfg, uint64_t tile_bytes) {
         if (cfg->order == SL_DYN) return 16u << 10;
         return tile_bytes >= 32u << 10 ? 32u << 10 : 0;
     case SL_CPASYNC:
-        if (tile_bytes < (cfg->order == SL_DYN ? 16u << 10 : 32u << 10)) return 0;
-        return static_cast<uint32_t>(std::min<uint64_t>(tile_bytes, 32u << 10));
+        return tile_bytes >= 16u << 10 ? static_cast<uint32_t>(std::min<uint64_t>(tile_bytes, 32u << 10)) : 0;
     case SL_TMA: return cfg->tma_ring == SL_RING_CTA ? 32u << 10 : 0;
     default: return 0;
     }
@@ -493,7 +496,7 @@ int make_plan(DevCtx* c, const void* buf, uint64_t bytes, int32_t dtype, const s
     // CTAs with at least one tile (the per-warp TMA ring deals tiles to warps)
     const uint64_t per_cta = cfg->mech == SL_TMA && cfg->tma_ring == SL_RING_WARP ? cta / 32 : 1;
     a.active = static_cast<uint32_t>(std::min<uint64_t>(grid, (total + per_cta - 1) / per_cta));
-    p->prefetch = first_bytes(cfg, tile_bytes);
+    p->prefetch = first_bytes(cfg, tile_bytes, grid < static_cast<int64_t>(p->resident) * c->info.sm_count);
     a.nst = cfg->mech == SL_TMA ? cfg->stages : 0;
     a.debug = cfg->debug_flags;
     a.timeout_ns = (cfg->debug_flags & SL_DEBUG_TMA_SKIP_STAGE) ? DEBUG_TIMEOUT_NS : TIMEOUT_NS;
