@@ -42,9 +42,8 @@ __global__ void __launch_bounds__(D * G > 8 ? 512 : 1024) k_cpasync_dyn(const KA
         len = left < chunk_vec ? static_cast<uint32_t>(left) : chunk_vec;
         p = buf + base + threadIdx.x;
     };
-    // (groups of copies folded together in the kernels that 128 registers are
-    // left to: 3 x 4 copies take 98 instead of 64, half the CTAs)
-    constexpr bool BIAS = BIASED<DT, G> && (D * G >= 16);
+    // (as in k_cpasync)
+    constexpr bool BIAS = BIASED<DT, G> && (D * G > 8);
     Acc<DT, BIAS> acc;
     uint32_t full_tiles = 0;
     volatile uint32_t* vs = slot;
