@@ -307,9 +307,9 @@ int sl_sweep(const void* dev_buf, uint64_t bytes, int32_t dtype, const sl_config
              sl_result* out);
 
 /* End-to-end form: the payload is in HOST memory (page-locked for full
- * speed).  Staged mode (cfg->host_direct == 0): up to 64 MiB, copies it to a
+ * speed).  Staged mode (cfg->host_direct == 0): up to 112 MiB, copies it to a
  * library-owned device staging buffer in one piece; above, to a staging ring in
- * chunks of 64 to 256 MiB on a copy stream, overlapped with the load kernel on
+ * two or more near-equal chunks of 48 to 256 MiB on a copy stream, overlapped with the load kernel on
  * each chunk, then combines all chunks.  Direct mode
  * (cfg->host_direct != 0): one load kernel reads the host buffer in place
  * through its device mapping (SL_ERR_ARG if the device cannot address it).

@@ -37,7 +37,8 @@ using sl::WarpPartial;
 
 constexpr int MAX_DEVICES = 64;
 constexpr uint64_t HOST_CHUNK = 256ull << 20;     // sl_run_host staging buffer
-constexpr uint64_t HOST_ONE = 64ull << 20;        // ... payloads up to this are not cut
+constexpr uint64_t HOST_ONE = 112ull << 20;       // ... payloads up to this are not cut
+constexpr uint64_t HOST_PIECE = 48ull << 20;      // ... others into pieces of at least this
 constexpr uint64_t TIMEOUT_NS = 2000000000ull;     // per-wait bound, normal runs
 constexpr uint64_t DEBUG_TIMEOUT_NS = 50000000ull;  // per-wait bound, fault-injection runs
 constexpr int64_t MAX_GRID = 1 << 20;
@@ -997,14 +998,21 @@ int sl_run_host(const void* host_buf, uint64_t bytes, int32_t dtype, const sl_co
         }
         CUDA_TRY(cudaStreamCreateWithFlags(&c->copy_stream, cudaStreamNonBlocking));
     }
-    // Up to 64 MiB the payload is copied in one piece on the caller's own stream
+    // Up to 112 MiB the payload is copied in one piece on the caller's own stream
     // and its kernel combines by itself, as sl_run's does: a chunk on the copy
     // stream costs about 8 us in events between the streams, more than the
     // kernel it would hide (256 KiB: 36 us by chunks and a combine kernel, 25 so;
-    // 1 MiB: 60 / 35; 64 MiB: 362 / 353, in eight chunks 373).  Above, in four
-    // chunks of at least 64 MiB (128 MiB: 683 us, 691 in eight), so that only the
-    // last one's kernel is not hidden behind the link.
-    const uint64_t step = std::min(HOST_CHUNK, std::max(HOST_ONE, (bytes / 4 + (1u << 20) - 1) >> 20 << 20));
+    // 1 MiB: 60 / 35; 64 MiB: 354, in two 360, in four 363; 96 MiB: 515 / 520 / 524).
+    // Above, in two to four near-equal chunks of at least 48 MiB, more only where
+    // a staging buffer would not hold them, so that the last one's kernel alone is
+    // not hidden behind the link (one / two / three / four pieces: 112 MiB 599.5 /
+    // 601.0 / 601.8 / 603.6 us, 128 MiB 684 / 680 / 682 / 686, 160 MiB 845 / 844 / 844 /
+    // 842, 192 MiB 1,008 / 1,006 / 1,005 / 1,001, 256 MiB 1,332 / 1,328 / 1,325 / 1,326; six and
+    // eight are slower again up to 512 MiB).
+    const uint64_t pieces = bytes <= HOST_ONE ? 1
+                                              : std::max(std::min<uint64_t>(4, bytes / HOST_PIECE),
+                                                         (bytes + HOST_CHUNK - 1) / HOST_CHUNK);
+    const uint64_t step = (bytes / pieces + (1u << 20) - 1) >> 20 << 20;
     const uint64_t chunk = std::min<uint64_t>(bytes, step);
     const uint64_t nchunks = bytes == 0 ? 0 : (bytes + step - 1) / step;
     // One launch shape for every chunk (planned on a full chunk), so every
