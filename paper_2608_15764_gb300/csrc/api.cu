@@ -555,6 +555,17 @@ const void* coverage_fn(const sl_config* cfg) {
     }
 }
 
+// Whether buf is memory of this context's device (not host or managed memory,
+// nor another device's).
+bool in_device_memory(const DevCtx* c, const void* buf) {
+    cudaPointerAttributes pa;
+    if (cudaPointerGetAttributes(&pa, buf) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    return pa.type == cudaMemoryTypeDevice && pa.device == c->dev;
+}
+
 int enqueue_locked(DevCtx* c, const void* buf, uint64_t bytes, int32_t dtype, const sl_config* cfg,
                    sl_result* dev_out, bool events, Plan* plan_out, uint32_t* cov = nullptr,
                    LaunchMode mode = LAUNCH_PLAIN) {
@@ -591,6 +602,14 @@ int enqueue_locked(DevCtx* c, const void* buf, uint64_t bytes, int32_t dtype, co
     p.args.done = sl::ctrl_done(c->err);
     p.args.result = dev_out;  // the kernel's last CTA writes the result
     if (cfg->order == SL_DYN) p.args.next = sl::ctrl_next(c->err);
+    if (mode == LAUNCH_WAIT) {
+        // ld.global.nc is for memory that nothing writes while the kernel runs, and
+        // a dependent launch runs from before the previous kernel's end
+        if (cfg->mech == SL_LDG && cfg->cop == SL_COP_NC_NA_L2_256) mode = LAUNCH_PLAIN;
+        // bytes prefetched before the wait are good only where this device's L2
+        // is also where whatever is still running writes: in its own memory
+        else if (p.prefetch && !in_device_memory(c, buf)) p.prefetch = 0;
+    }
     if (cfg->flush_l2) CUDA_TRY(sl::launch_flush(c->flush, c->flush_bytes / 16, c->info.sm_count, s));
     if (events) CUDA_TRY(cudaEventRecord(c->ev0, s));
     rc = launch(p, s, mode);
