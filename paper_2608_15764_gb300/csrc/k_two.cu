@@ -87,7 +87,7 @@ __global__ void __launch_bounds__(1024, 1) k_two(const TwoArgs t) {
 // One CTA of 64 threads: warp s reduces stream s's warp partials (CTA-major,
 // exact integer sums and XOR), lane 0 writes {sum, xor, issued} of the stream
 // to out[3s..3s+2]; out[6..10] take the five timer words.
-__global__ void __launch_bounds__(64) k_two_combine(const TwoArgs t, uint32_t grid, uint64_t* out) {
+__global__ void __launch_bounds__(64, 1) k_two_combine(const TwoArgs t, uint32_t grid, uint64_t* out) {
     const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t w0 = warp ? t.warps_a : 0u;
     const uint32_t nw = warp ? t.warps_b : t.warps_a;
