@@ -58,6 +58,20 @@ __device__ __forceinline__ WarpPartial warp_partial(const Acc<DT, BIAS>& acc) {
     return p;
 }
 
+// The block's and the grid's size, as tid_here: what is computed from the thread's
+// place is kept out of the registers through stream() below, ten of them in an LDG
+// kernel (K = 4 uint32 42 -> 33, K = 16 102 -> 81).
+__device__ __forceinline__ uint32_t threads_here() {
+    uint32_t t;
+    asm volatile("mov.u32 %0, %%ntid.x;" : "=r"(t));
+    return t;
+}
+__device__ __forceinline__ uint32_t grid_here() {
+    uint32_t t;
+    asm volatile("mov.u32 %0, %%nctaid.x;" : "=r"(t));
+    return t;
+}
+
 // The item loop of a class kernel whose CTAs work on one item together.
 // stream(item) folds an item and returns the warp's partial.  The next item's descriptor is copied to
 // shared memory, and the one after it claimed, while the current item streams;
@@ -73,20 +87,6 @@ __device__ __forceinline__ WarpPartial warp_partial(const Acc<DT, BIAS>& acc) {
 // thread 0 writes index j + 3, so there are four index words (with three,
 // index j + 3 would be index j's); they read descriptor j + 1 and partials j
 // while descriptor j + 2 and partials j + 1 are written: two of each.
-// What is computed from the thread's place is kept out of the registers through
-// stream() (tid_here; the same for the block's and the grid's size): ten registers
-// in an LDG kernel (K = 4 uint32 42 -> 33, K = 16 102 -> 81).
-__device__ __forceinline__ uint32_t threads_here() {
-    uint32_t t;
-    asm volatile("mov.u32 %0, %%ntid.x;" : "=r"(t));
-    return t;
-}
-__device__ __forceinline__ uint32_t grid_here() {
-    uint32_t t;
-    asm volatile("mov.u32 %0, %%nctaid.x;" : "=r"(t));
-    return t;
-}
-
 template <bool FLOATS, typename Stream>
 __device__ __forceinline__ void batch_items(const BArgs& a, Stream stream) {
     __shared__ BatchItem slot[2];
