@@ -132,8 +132,10 @@ int plan_ctas(const void* fn, const Group& g, int sms, int* ctas, const char** w
     if (!cuda_ok(cudaFuncGetAttributes(&fa, fn), "cudaFuncGetAttributes failed")) return status;
     if (fa.localSizeBytes > 0) return infeasible("tuning entry: kernel spills registers");
     if (g.block > fa.maxThreadsPerBlock) return infeasible("tuning entry: too many threads for this kernel");
-    if (g.smem > 0 && !cuda_ok(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                    static_cast<int>(g.smem)), "cudaFuncSetAttribute failed"))
+    // (raised, never lowered: classes with other rings, and other batches, launch this kernel too)
+    if (static_cast<int>(g.smem) > fa.maxDynamicSharedSizeBytes &&
+        !cuda_ok(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(g.smem)),
+                 "cudaFuncSetAttribute failed"))
         return status;
     int res = 0;
     if (!cuda_ok(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&res, fn, g.block, g.smem), "occupancy query failed"))
