@@ -425,8 +425,8 @@ typedef struct sl_batch sl_batch;  /* opaque */
  * persistent kernel per size class streaming many uneven buffers, in one
  * CUDA-graph launch; no paper counterpart).  Each buffer goes to the first
  * table entry that matches it (SL_ERR_ARG if none).  Buffers are cut into
- * work items (a part of a CTA's share of its class, at most 256 KiB; TMA
- * classes 128 KiB to 1 MiB); each class kernel runs a persistent grid whose
+ * work items (a part of a CTA's share of its class, at most 256 KiB, 1 MiB where
+ * few CTAs share an SM; TMA classes 128 KiB to 1 MiB); each class kernel runs a persistent grid whose
  * CTAs claim items from an atomic counter, fold them with the class's
  * mechanism and write the item's partials (one; TMA classes one per warp); a
  * combine kernel with one CTA per buffer adds each buffer's partials (integer

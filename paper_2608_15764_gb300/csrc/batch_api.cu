@@ -219,13 +219,21 @@ int plan_group(Group& g, int sms, int smem_optin) {
 // partial each at the end of every item: an item is a CTA's share there, at
 // least 128 KiB (64 buffers, 1 GiB, four types: 243 us in items of a sixth of the
 // share, 190 so) and at most 1 MiB (16 GiB of bfloat16: 2,558 us, 2,610 in
-// 256 KiB items).  256 KiB is enough for the others.
-constexpr uint64_t ITEM_MAX = 256ull << 10, ITEM_TMA_MIN = 128ull << 10, ITEM_TMA_MAX = 1ull << 20;
+// 256 KiB items).  256 KiB is enough for the others, whose loads or copies drain at
+// the end of an item, where the other CTAs of the SM cover that: with one, two, ... CTAs
+// on an SM an item may have 16, 8, ... units, up to 1 MiB (16 GiB by LDG K = 12 at 512
+// threads, one CTA per SM, in 256 KiB / so: uint32 2,579 / 2,243 us, bfloat16
+// 2,896 / 2,383; K = 8 at 512 FP32 2,471 / 2,342, FP8 2,684 / 2,489; twice as many units are
+// 2-6% slower over 1 GiB).
+constexpr uint64_t ITEM_MAX = 256ull << 10, ITEM_FEW = 1ull << 20, ITEM_TMA_MIN = 128ull << 10;
+constexpr uint64_t ITEM_UNITS = 16;
 
-uint64_t item_bytes(const Group& g) {
+uint64_t item_bytes(const Group& g, int sms) {
     const bool tma = g.cfg.mech == SL_TMA;
     const uint64_t share = g.bytes / ((tma ? 1 : 4) * static_cast<uint64_t>(g.ctas));
-    const uint64_t want = tma ? std::min(std::max(share, ITEM_TMA_MIN), ITEM_TMA_MAX) : std::min(share, ITEM_MAX);
+    const uint64_t few = ITEM_UNITS / std::max<uint64_t>(1, static_cast<uint64_t>(g.ctas / sms)) * g.unit;
+    const uint64_t want = tma ? std::min(std::max(share, ITEM_TMA_MIN), ITEM_FEW)
+                              : std::min(share, std::min(std::max(ITEM_MAX, few), ITEM_FEW));
     return g.unit * std::max<uint64_t>(1, want / g.unit);
 }
 
@@ -303,7 +311,7 @@ int build_batch(sl_batch* b, const sl_batch_desc* descs, int32_t n, const sl_tun
     for (int32_t i = 0; i < n; ++i) {
         Group& g = b->groups[b->class_of[i]];
         first[i] = g.items.size();
-        const uint64_t bytes = descs[i].bytes, step = item_bytes(g);
+        const uint64_t bytes = descs[i].bytes, step = item_bytes(g, sms);
         const uint8_t* p = static_cast<const uint8_t*>(descs[i].ptr);
         for (uint64_t off = 0; off < bytes; off += step) {
             BatchItem it;
@@ -331,7 +339,7 @@ int build_batch(sl_batch* b, const sl_batch_desc* descs, int32_t n, const sl_tun
     std::vector<BufSeg> segs(n);
     for (int32_t i = 0; i < n; ++i) {
         const Group& g = b->groups[b->class_of[i]];
-        const uint64_t step = item_bytes(g);
+        const uint64_t step = item_bytes(g, sms);
         segs[i].pstart = static_cast<uint32_t>(g.part_off + first[i] * g.slots);
         segs[i].pcount = static_cast<uint32_t>((descs[i].bytes + step - 1) / step * g.slots);
     }
