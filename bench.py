@@ -421,7 +421,7 @@ def run_ours(a):
         return 0
 
     # ---- end to end through the public host-buffer entry point
-    # Staged: 64-256 MiB copies to device staging overlapped with the kernel on
+    # Staged: 48-256 MiB copies to device staging overlapped with the kernel on
     # the previous chunk.  Direct: one kernel reads the pinned host buffer in
     # place over the CPU-GPU link (longer latency: more bytes in flight).  The
     # faster measured mode is reported.
