@@ -269,8 +269,10 @@ int sl_run(const void* dev_buf, uint64_t bytes, int32_t dtype, const sl_config* 
  * fields are 0) to the DEVICE pointer dev_out (8-byte aligned).  Successive enqueues on one stream may share the
  * library's scratch; enqueues on different streams at once race.  The kernel
  * reads the buffer after everything before it on the stream, as an ordinary
- * launch would (outside a capture it is a programmatic dependent launch that
- * waits for the previous kernel, which shortens the gap between the two). */
+ * launch would (outside a capture, and but for SL_COP_NC_NA_L2_256, it is a
+ * programmatic dependent launch that waits for the previous kernel, which
+ * shortens the gap between the two; it may prefetch from the buffer before that,
+ * where the buffer is memory of this device). */
 int sl_enqueue(const void* dev_buf, uint64_t bytes, int32_t dtype, const sl_config* cfg,
                sl_result* dev_out);
 
