@@ -13,7 +13,7 @@ BYTES, NBUF, CHAIN = 48 << 20, 48, 16  # 48 buffers: none is in L2 when its turn
 
 
 @pytest.mark.parametrize("mech,kw", [("cpasync", dict(k=2, copies=8, cta=256)), ("ldg", dict(k=8, cta=256, order="dyn")),
-                                     ("tma", dict(cta=256, stage_bytes=16384, stages=2))])
+                                     ("tma", dict(cta=256, stage_bytes=16384, stages=4))])
 def test_window_of_a_chain(mech, kw):
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
